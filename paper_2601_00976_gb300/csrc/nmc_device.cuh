@@ -30,20 +30,115 @@ __device__ __forceinline__ float r_fma(float a, float b, float c) { return fmaf(
 __device__ __forceinline__ double r_log10(double x) { return log10(x); }
 __device__ __forceinline__ float r_log10(float x) { return log10f(x); }
 
+// Comparisons of FP64 values on the integer pipe.  An FP64 compare is an FP64-pipe instruction (~64
+// cycles of an SMSP's pipe, as any other), while non-negative doubles order like their bit patterns:
+// two integer instructions give the same answer.  kInfBits is +infinity's pattern; NaN patterns are
+// above it.
+constexpr unsigned long long kInfBits = 0x7ff0000000000000ull;
+
+__device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ unsigned long long abs_bits(double x) { return bits_of(x) & 0x7fffffffffffffffull; }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x7ff00000; }
+__device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
+// |a| > b for b >= 0 (false when either is NaN)
+__device__ __forceinline__ bool abs_gt(double a, double b) {
+    const unsigned long long ka = abs_bits(a);
+    return ka > bits_of(b) && ka <= kInfBits;
+}
+// fmax(|a|, |b|): a NaN operand yields the other one (0 when both are NaN)
+__device__ __forceinline__ double abs_max(double a, double b) {
+    unsigned long long ka = abs_bits(a), kb = abs_bits(b);
+    if (ka > kInfBits) ka = 0;
+    if (kb > kInfBits) kb = 0;
+    return __longlong_as_double((long long)(ka > kb ? ka : kb));
+}
+// x <= t for x >= 0 or NaN (false) and t >= 0
+__device__ __forceinline__ bool nonneg_le(double x, double t) { return bits_of(x) <= bits_of(t); }
+__device__ __forceinline__ bool nonneg_le(float x, float t) { return x <= t; }
+
+// The largest t with sqrt(t) <= thr (square root rounded to nearest), thr >= 0: a test sqrt(u) <= thr
+// is then u <= t, without the square root (~12 FP64-pipe instructions in every warp of every inner
+// iteration).  sqrt rounds to thr or below for u up to (thr + ulp(thr) / 2)^2, which lies between
+// thr^2 and thr^2 + 2 ulp(thr^2), so t is fl(thr^2) or its successor; among denormals and at overflow
+// fl(thr^2) may itself be one step too large.
+__device__ __forceinline__ double next_bits(double x, int d) { return __longlong_as_double(__double_as_longlong(x) + d); }
+__device__ __forceinline__ float next_bits(float x, int d) { return __int_as_float(__float_as_int(x) + d); }
+template <typename T>
+__device__ __forceinline__ T square_threshold(T thr) {
+    T t = thr * thr;
+    if (r_sqrt(t) > thr) return next_bits(t, -1);
+    if (!is_finite(t)) return t;
+    const T n = next_bits(t, 1);
+    return r_sqrt(n) <= thr ? n : t;
+}
+
+// Warp sums of K values by recursive halving: at each step a lane keeps half of the values it still
+// carries and hands the other half to its partner, so K values cost ~K + 5 additions instead of the
+// 5 K of a butterfly per value (an FP64 addition holds the SMSP's pipe ~64 cycles: the three Gram
+// sums of an inner iteration 6 instead of 15, the velocity solve's fifteen sums 16 instead of 75).
+// Every value is added over the same tree as the butterfly adds it (partners 16, 8, 4, 2, 1 apart;
+// addition commutes), so the sums are the same bit for bit.  Together with the integer comparisons and
+// square_threshold above it took the FP64 solve of 20001 profile nodes (32 energies) from 89.3 to 77.1 ms,
+// the O(v/c) solve of 8192 nodes from 57.6 to 50.1 ms and the mixed solve of 200003 core/tail nodes from
+// 164.4 to 157.1 ms.  The sum a lane ends with in v[0] is that
+// of value fold_index<K>(lane) (K or more: none).
+template <int N, int OFF, typename T>
+__device__ __forceinline__ void fold_step(T* v, int lane) {
+    if constexpr (OFF > 0) {
+        if constexpr (N == 1) {
+            v[0] += __shfl_xor_sync(kFull, v[0], OFF);
+            fold_step<1, OFF / 2>(v, lane);
+        } else {
+            constexpr int H = (N + 1) / 2;
+            const bool up = (lane & OFF) != 0;
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                if (k + H < N) {
+                    const T keep = up ? v[k + H] : v[k], give = up ? v[k] : v[k + H];
+                    v[k] = keep + __shfl_xor_sync(kFull, give, OFF);
+                } else {
+                    v[k] += __shfl_xor_sync(kFull, v[k], OFF);
+                }
+            }
+            fold_step<H, OFF / 2>(v, lane);
+        }
+    }
+}
+
+template <int K>
+constexpr int kFoldLevels = 1 + kFoldLevels<(K + 1) / 2>;
+template <>
+constexpr int kFoldLevels<1> = 0;
+
+template <int K>
+__device__ __forceinline__ int fold_index(int lane) {
+    int base = 0, left = K, n = K;
+#pragma unroll
+    for (int l = 0; l < kFoldLevels<K>; ++l) {
+        const int h = (n + 1) / 2;
+        if (lane & (16 >> l)) { base += h; left -= h; }
+        else left = left < h ? left : h;
+        n = h;
+    }
+    return left >= 1 ? base : K;
+}
+
+// Warp w's sums of the K values to scratch[w * K + k].
+template <int K, typename T>
+__device__ __forceinline__ void warp_partials(T (&v)[K], void* scratch) {
+    static_assert(kFoldLevels<K> <= 5, "at most 32 values a warp");
+    T* red = static_cast<T*>(scratch);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    fold_step<K, 16>(v, lane);
+    const int k = fold_index<K>(lane);
+    if ((lane & ((32 >> kFoldLevels<K>) - 1)) == 0 && k < K) red[w * K + k] = v[0];
+}
+
 // Sum K values over the whole block; result in out[0..K).
 template <int K, typename T>
 __device__ __forceinline__ void block_sum(T (&v)[K], void* scratch, T* out) {
     T* red = static_cast<T*>(scratch);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(kFull, v[k], off);
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) red[w * K + k] = v[k];
-    }
+    warp_partials<K, T>(v, scratch);
     __syncthreads();
     if (threadIdx.x < K) {
         const int nw = blockDim.x >> 5;
@@ -103,24 +198,8 @@ __device__ __forceinline__ float f2_residual(F2 A, F2 c, F2 x, float t) {
     return __fadd_rn(__fadd_rn(s, t), __fadd_rn(e, __fsub_rn(A.l, pe)));
 }
 
-// block_sum split at its first barrier: warp w's sums of the K values land in
-// scratch[w * K + k]; after a barrier, sum_partials in any one thread adds the
-// warps' partials in the order block_sum uses.
-template <int K, typename T>
-__device__ __forceinline__ void warp_partials(T (&v)[K], void* scratch) {
-    T* red = static_cast<T*>(scratch);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(kFull, v[k], off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        const int w = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < K; ++k) red[w * K + k] = v[k];
-    }
-}
-
+// block_sum split at its first barrier: after warp_partials and a barrier, sum_partials in any one
+// thread adds the warps' partials in the order block_sum uses.
 template <int K, typename T>
 __device__ __forceinline__ void sum_partials(const void* scratch, T (&out)[K]) {
     const T* red = static_cast<const T*>(scratch);
@@ -168,6 +247,44 @@ __device__ __forceinline__ void species_sum(T (&v)[K], void* scratch, T* out, in
         }
         __syncthreads();
     }
+}
+
+// Algorithm 2: v holds the thread's weighted squares of the change of its bin's four moments; true in
+// every thread of a warp's lanes together exactly when each species' sums pass their tests, number
+// moment v[0] against t2_d[s] and the first moments against t2_i[s] (square_threshold values).  The
+// sums are formed by recursive halving, so a lane ends with one moment's sum of its species and votes
+// on that one; the caller combines the votes over the block.  Species spanning several warps meet at a
+// barrier of that species' warps only (named barrier 1 + s; barrier 0 is the block's) and use `scratch`,
+// which must be free from the previous block barrier on.
+template <typename T>
+__device__ __forceinline__ int species_vote(T (&v)[4], const T* t2_d, const T* t2_i, int nep, int ns, int s,
+                                            void* scratch) {
+    const int lane = threadIdx.x & 31;
+    if (nep <= 32) {
+        int off = nep >> 1;   // nep >= 2
+        const bool up = (lane & off) != 0;
+        const T a = (up ? v[2] : v[0]) + __shfl_xor_sync(kFull, up ? v[0] : v[2], off);
+        const T b = (up ? v[3] : v[1]) + __shfl_xor_sync(kFull, up ? v[1] : v[3], off);
+        off >>= 1;
+        const int sp = s < ns ? s : 0;
+        bool ok;
+        if (off == 0) {
+            ok = nonneg_le(a, up ? t2_i[sp] : t2_d[sp]) && nonneg_le(b, t2_i[sp]);
+        } else {
+            const bool up2 = (lane & off) != 0;
+            T x = (up2 ? b : a) + __shfl_xor_sync(kFull, up2 ? a : b, off);
+            for (off >>= 1; off > 0; off >>= 1) x += __shfl_xor_sync(kFull, x, off);
+            ok = nonneg_le(x, up || up2 ? t2_i[sp] : t2_d[sp]);
+        }
+        return s < ns ? (int)ok : 1;
+    }
+    const int wps = nep >> 5, w = threadIdx.x >> 5, c = lane & 3;
+    T* pv = static_cast<T*>(scratch);
+    warp_partials<4, T>(v, scratch);
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + s), "r"(wps * 32) : "memory");
+    T u = 0;
+    for (int i = 0; i < wps; ++i) u += pv[(s * wps + i) * 4 + c];
+    return nonneg_le(u, c == 0 ? t2_d[s] : t2_i[s]);
 }
 
 // Cell index and fractional offset of v on a uniform axis, clamped to the
@@ -286,18 +403,18 @@ __device__ __forceinline__ void anderson3_warp(double e, int n, double& c0, doub
     c1 = 0.0;
     cL = 1.0;
     if (n == 1) {
-        if (fabs(a00) > 1e-14 * fabs(a00) && isfinite(a00)) {
+        if (abs_bits(a00) - 1 < kInfBits - 1) {   // |a00| > 1e-14 |a00| and finite: neither 0, infinite nor NaN
             const double gam = r0 / a00;
-            if (isfinite(gam)) { c0 = gam; cL = 1.0 - gam; }
+            if (is_finite(gam)) { c0 = gam; cL = 1.0 - gam; }
         }
     } else if (n == 2) {
-        const double dmax = fmax(fabs(a00), fabs(a11));
-        if (dmax > 0.0 && isfinite(dmax)) {
+        const double dmax = abs_max(a00, a11);
+        if (bits_of(dmax) - 1 < kInfBits - 1) {   // dmax > 0 and finite
             // column 0 with partial pivoting (A is symmetric: a10 = a01)
-            const bool sw = fabs(a01) > fabs(a00);
+            const bool sw = abs_gt(a01, __longlong_as_double((long long)abs_bits(a00)));
             const double p0 = sw ? a01 : a00, p1 = sw ? a11 : a01, pr = sw ? r1 : r0;
             const double q0 = sw ? a00 : a01, q1 = sw ? a01 : a11, qr = sw ? r0 : r1;
-            if (fabs(p0) > 1e-14 * dmax) {
+            if (abs_gt(p0, 1e-14 * dmax)) {
                 // lane 0: det = p0 q1 - q0 p1; lane 1: p0 qr - q0 pr (gamma1 det);
                 // lane 2: pr q1 - p1 qr (gamma0 det), as one x y - z w
                 const double x = lane == 2 ? pr : p0;
@@ -306,11 +423,11 @@ __device__ __forceinline__ void anderson3_warp(double e, int n, double& c0, doub
                 const double w = lane == 0 ? p1 : (lane == 1 ? pr : qr);
                 const double t = x * y - z * w;
                 const double det = __shfl_sync(kFull, t, 0);
-                if (fabs(det) > 1e-14 * dmax * fabs(p0)) {
+                if (abs_gt(det, 1e-14 * dmax * fabs(p0))) {
                     const double gm = t * (1.0 / det);
                     const double gm1 = __shfl_sync(kFull, gm, 1), gm0 = __shfl_sync(kFull, gm, 2);
                     const double sum = gm0 + gm1;
-                    if (isfinite(sum)) { c0 = gm0; c1 = gm1; cL = 1.0 - sum; }
+                    if (is_finite(sum)) { c0 = gm0; c1 = gm1; cL = 1.0 - sum; }
                 }
             }
         }
@@ -419,11 +536,11 @@ struct OpacState {
     double eta_e;              // mu_e / T
     double mu[kMaxSpecies];    // neutrino chemical potentials per species
     double tinv;               // 1 / T
-    double tr, tt, ty, kt, ke; // fractional offsets in the table cells
+    double w8[8], w4[4];       // corner weights of the EmAb/Iso cell (bits: rho, T, Ye) and the kernel cell (T, eta)
     double pre[4];             // dtau sc_EmAb, dtau sc_Iso, and the NES and pair prefactors
     // FP32 copies for the mixed-precision path: mu and 1 / T as double-floats
     float mu_h[kMaxSpecies], mu_l[kMaxSpecies], tinv_h, tinv_l;
-    float wf[5];               // tr, tt, ty, kt, ke
+    float w8_f[8], w4_f[4];
     float pre_f[4];
     int ir, it, iy, ikt, ike;  // table cells
 };
@@ -505,12 +622,19 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
         double ct = 0.0;
         axis_cell<double>(ln == 0 ? lrho : ((ln == 1 || ln == 3) ? lT : (ln == 2 ? Ye : eta_e)), ax, &ci, &ct, &cl);
         const bool any_cl = __ballot_sync(kFull, cl && ln < nax) != 0u;
-        if (ln == 0) { os->ir = ci; os->tr = ct; }
-        if (ln == 1) { os->it = ci; os->tt = ct; }
-        if (ln == 2) { os->iy = ci; os->ty = ct; }
-        if (ln == 3 && nax == 5) { os->ikt = ci; os->kt = ct; }
-        if (ln == 4 && nax == 5) { os->ike = ci; os->ke = ct; }
-        if (kMixed && ln < nax) os->wf[ln] = (float)ct;
+        if (ln == 0) os->ir = ci;
+        if (ln == 1) os->it = ci;
+        if (ln == 2) os->iy = ci;
+        if (ln == 3 && nax == 5) os->ikt = ci;
+        if (ln == 4 && nax == 5) os->ike = ci;
+        {   // the tensor-product weights, one corner per lane, for every thread of the block
+            const R f0 = (R)__shfl_sync(kFull, ct, 0), f1 = (R)__shfl_sync(kFull, ct, 1), f2 = (R)__shfl_sync(kFull, ct, 2);
+            const R f3 = (R)__shfl_sync(kFull, ct, 3), f4 = (R)__shfl_sync(kFull, ct, 4);
+            const R w3 = ((ln & 1) ? f0 : (R)1 - f0) * ((ln & 2) ? f1 : (R)1 - f1) * ((ln & 4) ? f2 : (R)1 - f2);
+            const R w2 = ((ln & 1) ? f3 : (R)1 - f3) * ((ln & 2) ? f4 : (R)1 - f4);
+            if (ln < 8) { if constexpr (kMixed) os->w8_f[ln] = w3; else os->w8[ln] = w3; }
+            if (ln < 4) { if constexpr (kMixed) os->w4_f[ln] = w2; else os->w4[ln] = w2; }
+        }
         if (ln == 0) {
             os->tinv = tinv;
             os->eta_e = eta_e;
@@ -565,6 +689,7 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
 #pragma unroll
                 for (int u = 0; u < kFdBatch; ++u) {
                     const int k = k0 + u * nthr;
+                    if (k >= nfdp) break;   // a batch is seldom full: no exponentials past the last point
                     const int sf = k >= 2 * nqp ? 2 : (k >= nqp ? 1 : 0);
                     const int i = k - sf * nqp;
                     R fv, fcv = 0;
@@ -590,7 +715,7 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
                         const R mu = (R)os->mu[sf];
                         fv = (R)1 / (r_exp((eh[u] - mu) * Tinv) + (R)1);
                     }
-                    if (k < nfdp && NMC_IN_BOUNDS(g.dbg, (long long)((kMixed ? NS : 0) + sf) * nqp + i,
+                    if (NMC_IN_BOUNDS(g.dbg, (long long)((kMixed ? NS : 0) + sf) * nqp + i,
                                                   (long long)(kMixed ? 2 : 1) * NS * nqp, kDbgSmemFd)) {
                         fq[sf * nqp + i] = fv;
                         if constexpr (kMixed) fq[(NS + sf) * nqp + i] = fcv;
@@ -669,8 +794,9 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
                 if (vmax > dmax) theta = fmin(theta, (dmax - avg) / (vmax - avg));
 #pragma unroll
                 for (int pp = 0; pp < kMaxNq; ++pp) {
+                    if (pp >= nq) break;
                     coef[pp] = avg + theta * (coef[pp] - avg);
-                    coefc[pp] = avgc + theta * (coefc[pp] - avgc);
+                    if (kMixed) coefc[pp] = avgc + theta * (coefc[pp] - avgc);
                 }
                 // the limiter puts the extreme point on the bound in exact arithmetic; the rounding of
                 // avg + theta (v - avg) can leave it just outside (below zero where avg is far above
@@ -679,8 +805,9 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
                 const R cmin = (R)(1.0 - P.d_max), cmax = (R)(1.0 - P.d_min);
 #pragma unroll
                 for (int pp = 0; pp < kMaxNq; ++pp) {
+                    if (pp >= nq) break;
                     coef[pp] = coef[pp] < dmin ? dmin : (coef[pp] > dmax ? dmax : coef[pp]);
-                    coefc[pp] = coefc[pp] < cmin ? cmin : (coefc[pp] > cmax ? cmax : coefc[pp]);
+                    if (kMixed) coefc[pp] = coefc[pp] < cmin ? cmin : (coefc[pp] > cmax ? cmax : coefc[pp]);
                 }
             }
 #pragma unroll
@@ -689,7 +816,7 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
                 const int sq = s * NEP + e * nq + pp;
                 const R dc = kMixed ? coefc[pp] : (R)1 - coef[pp];
                 b.vDeq[sq] = coef[pp];
-                b.vDeqc[sq] = coefc[pp];
+                if (kMixed) b.vDeqc[sq] = coefc[pp];
                 b.vA[sq] = coef[pp] / dc;
                 b.vAi[sq] = dc / coef[pp];
             }
@@ -706,9 +833,6 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
         const long long dR = NE, dT = (long long)nr * NE, dY = (long long)nt * nr * NE;
         const bool tab_ok = NMC_IN_BOUNDS(g.dbg, base, tb.n_op, kDbgEmabIso) &&
                             NMC_IN_BOUNDS(g.dbg, base + dR + dT + dY, tb.n_op, kDbgEmabIso);
-        const R tr = kMixed ? (R)os->wf[0] : (R)os->tr;
-        const R tt = kMixed ? (R)os->wf[1] : (R)os->tt;
-        const R ty = kMixed ? (R)os->wf[2] : (R)os->ty;
         // ln chi as the first corner plus weighted differences: the corners are ~ -20, so an
         // FP32 sum of the corner values themselves would round ln chi by ~2e-6 in steps
         const R le0 = !tab_ok ? (R)0 : (kMixed ? (R)tb.emab_f[base] : (R)tb.emab[base]);
@@ -718,7 +842,7 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
         for (int c8 = 1; c8 < 8; ++c8) {
             if (!tab_ok) break;
             const int ca = c8 & 1, cb = (c8 >> 1) & 1, cc = c8 >> 2;
-            const R w = (ca ? tr : (R)1 - tr) * (cb ? tt : (R)1 - tt) * (cc ? ty : (R)1 - ty);
+            const R w = kMixed ? (R)os->w8_f[c8] : (R)os->w8[c8];
             const long long o = base + ca * dR + cb * dT + cc * dY;
             if (kMixed) { le += w * ((R)tb.emab_f[o] - le0); li += w * ((R)tb.iso_f[o] - li0); }
             else { le += w * ((R)tb.emab[o] - le0); li += w * ((R)tb.iso[o] - li0); }
@@ -732,10 +856,8 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
     }
     // NES and pair kernels: bilinear in (log10 T, eta_e), times dtau 4 pi / (hc)^3
     if (nes_on || pair_on) {
-        const R kt = kMixed ? (R)os->wf[3] : (R)os->kt;
-        const R ke = kMixed ? (R)os->wf[4] : (R)os->ke;
-        const R w00 = ((R)1 - kt) * ((R)1 - ke), w10 = kt * ((R)1 - ke);
-        const R w01 = ((R)1 - kt) * ke, w11 = kt * ke;
+        const R w00 = kMixed ? (R)os->w4_f[0] : (R)os->w4[0], w10 = kMixed ? (R)os->w4_f[1] : (R)os->w4[1];
+        const R w01 = kMixed ? (R)os->w4_f[2] : (R)os->w4[2], w11 = kMixed ? (R)os->w4_f[3] : (R)os->w4[3];
         const long long mat = (long long)NE * NE;
         const long long sE = mat, sT = (long long)tb.eta.n * mat;
         // One kernel order (Phi_0, or Phi_1 into PH1/AN1), as a list of jobs per lane of the species

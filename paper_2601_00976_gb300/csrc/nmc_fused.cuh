@@ -74,8 +74,8 @@ struct NodeShared {
     double G[MAXM][MAXM];
     double alpha[MAXM];
     float alpha_f[MAXM];
-    double thr[2][kMaxSpecies];   // Algorithm 2 thresholds on the D and I changes (FP64 path)
-    float thr_f[2][kMaxSpecies];  // the same rounded to FP32 (mixed path)
+    double t2[kMaxSpecies];       // Algorithm 2's thresholds on the squared changes (square_threshold; FP64 path)
+    float t2_f[2][kMaxSpecies];   // the same for the D and I changes of the mixed path, from FP32 thresholds
     double sp_out[kMaxSpecies * 4];
     double blk_out[8];
     OpacState op;
@@ -256,17 +256,18 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                 R v[1] = {Wt * M[0] * M[0]};
                 R* out = reinterpret_cast<R*>(nd->sp_out);
                 species_sum<1, R>(v, red, out, NEP, NS);
-                if (tid == lead) {
+                // one species per lane of the lead warp
+                const int sp = tid - lead;
+                if (sp >= 0 && sp < NS) {
                     const double fl = P.norm_floor * sqrt(g.sum_wt);
-                    // mixed precision: D is a double-float iterate held to tol_inner; the first
-                    // moments are FP32 values, checked against FP32 resolution at the finest
-                    const double tol_i = kMixed ? fmax(P.tol_inner, kFp32Resolution) : P.tol_inner;
-                    for (int sp = 0; sp < NS; ++sp) {
-                        const double dn = fmax((double)r_sqrt(out[sp]), fl);
-                        nd->thr[0][sp] = P.tol_inner * dn;
-                        nd->thr[1][sp] = tol_i * dn;
-                        nd->thr_f[0][sp] = (float)(P.tol_inner * dn);
-                        nd->thr_f[1][sp] = (float)(tol_i * dn);
+                    const double dn = fmax((double)r_sqrt(out[sp]), fl);
+                    if constexpr (kMixed) {
+                        // mixed precision: D is a double-float iterate held to tol_inner; the first
+                        // moments are FP32 values, checked against FP32 resolution at the finest
+                        nd->t2_f[0][sp] = square_threshold((float)(P.tol_inner * dn));
+                        nd->t2_f[1][sp] = square_threshold((float)(fmax(P.tol_inner, kFp32Resolution) * dn));
+                    } else {
+                        nd->t2[sp] = square_threshold(P.tol_inner * dn);
                     }
                 }
             }
@@ -576,50 +577,13 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c) { const R d = Mn[c] - M[c]; v[c] = Wt * d * d; }
                     if constexpr (kMixed) v[0] = Wt * sD * sD;
-                    if (act && !(isfinite(Mn[0]) && isfinite(Mn[1]) && isfinite(Mn[2]) && isfinite(Mn[3]) &&
-                                 isfinite(sD)))
+                    if (act && !(is_finite(Mn[0]) && is_finite(Mn[1]) && is_finite(Mn[2]) && is_finite(Mn[3]) &&
+                                 is_finite(sD)))
                         nd->bad = 1;
-                    auto species_ok = [&](const R* u, int sp) -> int {
-                        R mx = u[1];
-                        for (int c = 2; c < 4; ++c) mx = fmax(mx, u[c]);
-                        if constexpr (kMixed)
-                            return r_sqrt(u[0]) <= nd->thr_f[0][sp] && r_sqrt(mx) <= nd->thr_f[1][sp];
-                        else
-                            return r_sqrt(u[0]) <= nd->thr[0][sp] && r_sqrt(mx) <= nd->thr[1][sp];
-                    };
-                    if (NEP <= 32) {
-                        // a species group lies inside one warp: its sums are formed in registers
-                        // (the butterfly leaves the same sum in every lane of the group) and each
-                        // lane votes for its own species
-                        for (int off = NEP >> 1; off > 0; off >>= 1) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(kFull, v[c], off);
-                        }
-                        if (s < NS) vote = species_ok(v, s);
-                    } else {
-                        // a species spans NEP / 32 warps: warp sums by shuffles, then a barrier over that
-                        // species' warps only (named barrier 1 + s; barrier 0 is the block's), after which
-                        // every thread adds its species' partials in the same order and votes for it.  The
-                        // scratch is free here: the lead warp read the Gram partials before the previous
-                        // barrier, and the next ones are written after the vote's.
-                        const int wps = NEP >> 5, lane = tid & 31, w = tid >> 5;
-                        for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(kFull, v[c], off);
-                        }
-                        R* pv = reinterpret_cast<R*>(red);
-                        if (lane == 0) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) pv[w * 4 + c] = v[c];
-                        }
-                        asm volatile("bar.sync %0, %1;" ::"r"(1 + s), "r"(wps * 32) : "memory");
-                        R u[4] = {0, 0, 0, 0};
-                        for (int i = 0; i < wps; ++i) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) u[c] += pv[(s * wps + i) * 4 + c];
-                        }
-                        vote = species_ok(u, s);
-                    }
+                    // the scratch is free here: the lead warp read the Gram partials before the previous
+                    // barrier, and the next ones are written after the vote's
+                    if constexpr (kMixed) vote = species_vote(v, nd->t2_f[0], nd->t2_f[1], NEP, NS, s, red);
+                    else vote = species_vote(v, nd->t2, nd->t2, NEP, NS, s, red);
                 }
                 const bool conv = __syncthreads_and(vote) != 0;
                 const bool bad = *reinterpret_cast<volatile int*>(&nd->bad) != 0;
@@ -666,7 +630,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                                      fabs(yn1 - y1) <= P.tol_outer * fabs(nd->ystar[1]);   // Algorithm 3
                     int stop = conv, st = 0;
                     double Tn = nd->T;
-                    if (!(isfinite(yn0) && isfinite(yn1))) { st |= NMC_NONFINITE; stop = 1; }
+                    if (!(is_finite(yn0) && is_finite(yn1))) { st |= NMC_NONFINITE; stop = 1; }
                     if (!stop && k >= P.max_outer) { st |= NMC_NOT_CONVERGED_OUTER; stop = 1; }
                     if (!stop) {   // an iterate outside the EoS domain stops the node
                         bool ok;

@@ -55,7 +55,7 @@ struct VelNode {
     double qh[kMaxOuterMem][kNy], fh[kMaxOuterMem][kNy];
     double G[3][3];
     double alpha[3];
-    double thr[2][kMaxSpecies];
+    double t2[kMaxSpecies];               // Algorithm 2's thresholds on the squared changes
     double sp_out[kMaxSpecies * 4];
     double blk_out[16];
     OpacState op;
@@ -308,13 +308,10 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
             {   // reference norm ||D^[k,1]||_W per species and the Algorithm 2 thresholds
                 double v[1] = {Wt * M[0] * M[0]};
                 species_sum<1, double>(v, red, nd->sp_out, NEP, NS);
-                if (tid == lead) {
+                const int sp = tid - lead;   // one species per lane of the lead warp
+                if (sp >= 0 && sp < NS) {
                     const double fl = P.norm_floor * sqrt(g.sum_wt);
-                    for (int sp = 0; sp < NS; ++sp) {
-                        const double dn = fmax(sqrt(nd->sp_out[sp]), fl);
-                        nd->thr[0][sp] = P.tol_inner * dn;
-                        nd->thr[1][sp] = P.tol_inner * dn;
-                    }
+                    nd->t2[sp] = square_threshold(P.tol_inner * fmax(sqrt(nd->sp_out[sp]), fl));
                 }
             }
             auto publish = [&](const double (&Mv)[4]) {
@@ -450,21 +447,9 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                 {   // Algorithm 2
                     double v[4];
                     for (int c = 0; c < 4; ++c) { const double d = Mn[c] - M[c]; v[c] = Wt * d * d; }
-                    if (act && !(isfinite(Mn[0]) && isfinite(Mn[1]) && isfinite(Mn[2]) && isfinite(Mn[3])))
+                    if (act && !(is_finite(Mn[0]) && is_finite(Mn[1]) && is_finite(Mn[2]) && is_finite(Mn[3])))
                         nd->bad = 1;
-                    auto species_ok = [&](const double* u, int sp) -> int {
-                        double mx = u[1];
-                        for (int c = 2; c < 4; ++c) mx = fmax(mx, u[c]);
-                        return sqrt(u[0]) <= nd->thr[0][sp] && sqrt(mx) <= nd->thr[1][sp];
-                    };
-                    if (NEP <= 32) {
-                        for (int off = NEP >> 1; off > 0; off >>= 1)
-                            for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(kFull, v[c], off);
-                        if (s < NS) vote = species_ok(v, s);
-                    } else {
-                        species_sum<4, double>(v, red, nd->sp_out, NEP, NS);
-                        for (int sp = 0; sp < NS; ++sp) vote &= species_ok(nd->sp_out + sp * 4, sp);
-                    }
+                    vote = species_vote(v, nd->t2, nd->t2, NEP, NS, s, red);
                 }
                 const bool conv = __syncthreads_and(vote) != 0;
                 const bool bad = *reinterpret_cast<volatile int*>(&nd->bad) != 0;
@@ -501,7 +486,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                     int conv = 1, fin = 1;
                     for (int c = 0; c < kNy; ++c) {   // Algorithm 3
                         if (!(fabs(yn[c] - y[c]) * nd->ri[c] <= P.tol_outer)) conv = 0;
-                        if (!isfinite(yn[c])) fin = 0;
+                        if (!is_finite(yn[c])) fin = 0;
                     }
                     int stop = conv, st = 0;
                     double Tn = nd->T;
