@@ -382,6 +382,7 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
     if (rc == NMC_OK) rc = upload_quads(ctx, tb->emab, ns, tb->n_ye, tb->n_t, tb->n_rho, ne, &t.emab_q);
     if (rc == NMC_OK) rc = upload_quads(ctx, tb->iso, ns, tb->n_ye, tb->n_t, tb->n_rho, ne, &t.iso_q);
     t.n_quad = (long long)ns * tb->n_ye * tb->n_t * (tb->n_rho - 1) * (ne - 1);
+    if (rc == NMC_OK) rc = build_interp_tables(ctx, tb);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->nes, n_nes, kCW, &t.nes_f);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->pair, n_pair, kCW, &t.pair_f);
     if (rc == NMC_OK) {

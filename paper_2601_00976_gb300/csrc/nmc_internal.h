@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "nmc.h"
+#include "nmc_fixed.cuh"
 
 namespace nmc {
 
@@ -134,6 +135,20 @@ struct DevTables {
     long long n_quad;
 };
 
+// Fixed-point tables of opacity_interp (built by nmc_create when the ln tables and axes fit: every ln
+// value finite and at most kFixedMax, log axes within 10^+-150; quads is null otherwise).  quads[which]:
+// per [ns][nye][nt][nrho-1][ne-1] cell its four (rho, E) corners as Q53, in the order rho_i E_q,
+// rho_i E_q+1, rho_i+1 E_q, rho_i+1 E_q+1.  Energy cell q: lne = log2 eps_q (Q52); (log2 E - lne) << sh
+// times rec is the fraction as Q62.
+struct InterpTables {
+    FixedAxis rho, t;
+    const FixedTables* ft;
+    const ulonglong2* quads[2];
+    const int64_t* lne;
+    const uint64_t* rec;
+    const int* sh;
+};
+
 struct SolveArgs {
     DevGrid g;
     DevTables tb;
@@ -218,6 +233,7 @@ struct nmc_ctx {
     std::vector<double> edges, eps, w2, w3;
     nmc::DevGrid g{};
     nmc::DevTables tb{};
+    nmc::InterpTables fx{};
     // device allocations owned by the context
     std::vector<void*> allocations;
     int* queue = nullptr;
@@ -242,6 +258,7 @@ int launch_fused(nmc_ctx* ctx, const SolveArgs& a, cudaStream_t stream);
 int launch_opacity_interp(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                           const double* T, const double* Ye, const double* E, double* out,
                           cudaStream_t stream);
+int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb);
 int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                                 const double* T, const double* Ye, const double* E, double* out,
                                 cudaStream_t stream);
