@@ -128,8 +128,9 @@ struct DevTables {
     const float* nes_f;
     const float* pair_f;
     long long n_op, n_nes, n_pair;   // element counts of the EmAb/Iso, NES and pair tables
-    // opacity_interp_mixed: the FP32 ln tables regrouped per (rho, E) cell, one float4
-    // (rho_i E_q, rho_i+1 E_q, rho_i E_q+1, rho_i+1 E_q+1) per [ns][nye][nt][nrho-1][ne-1]
+    // opacity_interp_mixed: the FP32 ln tables regrouped per (T, rho, E) cell, two float4
+    // (rho_i E_q, rho_i+1 E_q, rho_i E_q+1, rho_i+1 E_q+1) at T_j and T_j+1 per
+    // [ns][nye][nt-1][nrho-1][ne-1]; n_quad cells
     const float4* emab_q;
     const float4* iso_q;
     long long n_quad;
@@ -144,6 +145,7 @@ struct InterpTables {
     FixedAxis rho, t;
     const FixedTables* ft;
     const ulonglong2* quads[2];
+    long long n_quad;
     const int64_t* lne;
     const uint64_t* rec;
     const int* sh;
@@ -259,6 +261,7 @@ int launch_opacity_interp(nmc_ctx* ctx, int which, int species, long long p, con
                           const double* T, const double* Ye, const double* E, double* out,
                           cudaStream_t stream);
 int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb);
+int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev);
 int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                                 const double* T, const double* Ye, const double* E, double* out,
                                 cudaStream_t stream);

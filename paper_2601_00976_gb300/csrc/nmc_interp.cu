@@ -18,9 +18,12 @@
 // first corner plus weighted differences (the corners are ~ -20, whose FP32
 // sum would round ln chi by ~2e-6 in steps), and an FP32 exp; inputs and
 // outputs stay FP64.  The energy axis is searched in a shared-memory copy of
-// ln eps.  The table copy is regrouped per (rho, E) cell, four corners to a
-// float4, so a point's 16 corner values take four 16-byte loads (four L2
-// sectors) rather than sixteen scattered words.
+// ln eps.  The table copy is regrouped per (T, rho, E) cell, eight corners to a
+// 32-byte sector, so a point's 16 corner values come from two L2 sectors (from
+// four with (rho, E) cells, which left the kernel at the L2's rate: 8.6 TB/s of
+// sectors for 2.1 TB/s of points), and two points a thread are in flight.
+// 8.4 M points: 0.168 ms before these and the integer conversions, 0.121 ms now
+// (2.8 TB/s of points, 41% of the copy rate).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -83,6 +86,27 @@ __global__ void opacity_interp_kernel(const DevGrid g, const DevTables tb, int w
     }
 }
 
+// Energy search of both forms.  A bisection is five or six dependent shared-memory loads; instead the
+// logarithm's position on [lo, hi] picks one of kBuckets entries that hold the cell one bucket below
+// (never above the right cell), and a short scan ends at the last cell whose lower node is <= le.
+constexpr int kBuckets = 256;   // the kernels' block size
+
+template <typename V>
+__device__ __forceinline__ int cell_by_bisection(const V* node, int ne, V le) {
+    int lo = 0, hi = ne - 1;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (node[mid] <= le) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+template <typename V>
+__device__ __forceinline__ int cell_from(const V* node, int ne, V le, int lo) {
+    while (lo < ne - 2 && node[lo + 1] <= le) ++lo;
+    return lo;
+}
+
 constexpr int64_t kOneQ63 = INT64_MAX;
 
 // Cell and fraction (Q63) of v on a uniform log10 axis, clamped to it (zero, negative, NaN: its lower end).
@@ -114,7 +138,7 @@ __device__ __forceinline__ void cell_lin_q(double v, const Axis& ax, int* i, int
     *t = (int64_t)(((m << e) << 1) >> 1);
 }
 
-__global__ void __launch_bounds__(256) opacity_interp_fixed_kernel(const DevGrid g, const DevTables tb, const InterpTables fx,
+__global__ void __launch_bounds__(kBuckets) opacity_interp_fixed_kernel(const DevGrid g, const DevTables tb, const InterpTables fx,
                                                                    int which, int species, long long p,
                                                                    const double* __restrict__ rho,
                                                                    const double* __restrict__ T,
@@ -125,6 +149,7 @@ __global__ void __launch_bounds__(256) opacity_interp_fixed_kernel(const DevGrid
     __shared__ int64_t lne[kMaxNe];
     __shared__ uint64_t rec[kMaxNe];
     __shared__ int sh[kMaxNe];
+    __shared__ unsigned char lut[kBuckets];
     const int NE = g.ne;
     for (int k = threadIdx.x; k < (int)(sizeof(FixedTables) / 4); k += blockDim.x)
         reinterpret_cast<uint32_t*>(&ft)[k] = reinterpret_cast<const uint32_t*>(fx.ft)[k];
@@ -133,6 +158,11 @@ __global__ void __launch_bounds__(256) opacity_interp_fixed_kernel(const DevGrid
         rec[q] = fx.rec[q];
         sh[q] = fx.sh[q];
     }
+    __syncthreads();
+    // buckets of 2^shift of the Q52 logarithm
+    const int64_t lo_e = lne[0], hi_e = lne[NE - 1];
+    const int shift = max(0, 56 - (int)__clzll(hi_e - lo_e));   // (hi_e - lo_e) >> shift < kBuckets
+    lut[threadIdx.x] = (unsigned char)cell_by_bisection(lne, NE, lo_e + ((int64_t)threadIdx.x - 1) * (int64_t(1) << shift));
     __syncthreads();
     const ulonglong2* __restrict__ tab = which == 0 ? fx.quads[0] : fx.quads[1];
     const long long nrc = tb.rho.n - 1, nec = NE - 1;
@@ -145,15 +175,11 @@ __global__ void __launch_bounds__(256) opacity_interp_fixed_kernel(const DevGrid
         cell_q(T[i], fx.t, ft, &it, &tt);
         cell_lin_q(Ye[i], tb.ye, &iy, &ty);
         int64_t le = log2_q52(E[i], ft);
-        le = le < lne[0] ? lne[0] : (le > lne[NE - 1] ? lne[NE - 1] : le);
-        int lo = 0, hi = NE - 1;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (lne[mid] <= le) lo = mid; else hi = mid;
-        }
+        le = le < lo_e ? lo_e : (le > hi_e ? hi_e : le);
+        const int lo = cell_from(lne, NE, le, (int)lut[(le - lo_e) >> shift]);
         const long long base = (((sp0 + iy) * tb.t.n + it) * nrc + ir) * nec + lo;
-        if (!NMC_IN_BOUNDS(g.dbg, base, tb.n_quad, kDbgEmabIso) ||
-            !NMC_IN_BOUNDS(g.dbg, base + dT + dY, tb.n_quad, kDbgEmabIso))
+        if (!NMC_IN_BOUNDS(g.dbg, base, fx.n_quad, kDbgEmabIso) ||
+            !NMC_IN_BOUNDS(g.dbg, base + dT + dY, fx.n_quad, kDbgEmabIso))
             continue;
         ulonglong2 c[4][2];   // the (T, Ye) corners k = cb + 2 cc of the (rho, E) cell
 #pragma unroll
@@ -225,6 +251,23 @@ int upload_fx(nmc_ctx* ctx, const T* host, size_t count, const T** dev) {
     return NMC_OK;
 }
 
+// (float)x and (double)x in integers, the same values bit for bit: a conversion instruction runs on the FP64
+// pipe (~64 cycles of an SMSP), and a point of the FP32 form needs five.  Values whose FP32 form is not a
+// normal number take the instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    if (((hi >> 20) & 0x7ffu) - 897u > 253u) return (float)x;
+    const uint64_t u = word_of(x);
+    const uint64_t t = u + 0x0fffffffull + ((u >> 29) & 1u);   // round to nearest, ties to even
+    return __uint_as_float(((unsigned)(t >> 29) - (896u << 23)) | (hi & 0x80000000u));
+}
+
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+    if (e - 1u > 253u) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
 __device__ __forceinline__ void cell_f(float v, const Axis& ax, int* i, float* t) {
     float x = (v - (float)ax.lo) * (float)ax.inv_d;
     if (!(x >= 0.0f)) x = 0.0f;
@@ -235,60 +278,104 @@ __device__ __forceinline__ void cell_f(float v, const Axis& ax, int* i, float* t
     *t = x - (float)c;
 }
 
-__global__ void __launch_bounds__(256) opacity_interp_mixed_kernel(const DevGrid g, const DevTables tb, int which,
-                                                                   int species, long long p,
-                                                                   const double* __restrict__ rho,
-                                                                   const double* __restrict__ T,
-                                                                   const double* __restrict__ Ye,
-                                                                   const double* __restrict__ E,
-                                                                   double* __restrict__ out) {
+// U points per thread and step, kPointStride apart, so that their loads are in flight together.
+template <int U>
+__global__ void __launch_bounds__(kBuckets) opacity_interp_mixed_kernel(const DevGrid g, const DevTables tb, int which,
+                                                                        int species, long long p,
+                                                                        const double* __restrict__ rho,
+                                                                        const double* __restrict__ T,
+                                                                        const double* __restrict__ Ye,
+                                                                        const double* __restrict__ E,
+                                                                        double* __restrict__ out) {
     __shared__ float lne[kMaxNe];
+    __shared__ unsigned char lut[kBuckets];
     const int NE = g.ne;
     for (int q = threadIdx.x; q < NE; q += blockDim.x) lne[q] = (float)g.lneps[q];
     __syncthreads();
+    const float lo_e = lne[0], hi_e = lne[NE - 1], per_bucket = (hi_e - lo_e) / kBuckets, scale = kBuckets / (hi_e - lo_e);
+    lut[threadIdx.x] = (unsigned char)cell_by_bisection(lne, NE, lo_e + ((int)threadIdx.x - 1) * per_bucket);
+    __syncthreads();
     const float4* __restrict__ tab = which == 0 ? tb.emab_q : tb.iso_q;
-    const long long nrc = tb.rho.n - 1, nec = NE - 1;
-    const long long dT = nrc * nec, dY = (long long)tb.t.n * nrc * nec;
-    const long long sp0 = (long long)species * tb.ye.n;
-    const float lo_e = lne[0], hi_e = lne[NE - 1];
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p; i += (long long)gridDim.x * blockDim.x) {
-        int ir, it, iy;
-        float tr, tt, ty;
-        cell_f(log10f((float)rho[i]), tb.rho, &ir, &tr);
-        cell_f(log10f((float)T[i]), tb.t, &it, &tt);
-        cell_f((float)Ye[i], tb.ye, &iy, &ty);
-        float le = logf((float)E[i]);
-        if (!(le >= lo_e)) le = lo_e;
-        if (le > hi_e) le = hi_e;
-        int lo = 0, hi = NE - 1;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (lne[mid] <= le) lo = mid; else hi = mid;
-        }
-        const float te = (le - lne[lo]) / (lne[lo + 1] - lne[lo]);
-        // the (rho, E) cell's four corners per load: (T, Ye) corners k = cb + 2 cc
-        const long long base = (((sp0 + iy) * tb.t.n + it) * nrc + ir) * nec + lo;
-        if (!NMC_IN_BOUNDS(g.dbg, base, tb.n_quad, kDbgEmabIso) ||
-            !NMC_IN_BOUNDS(g.dbg, base + dT + dY, tb.n_quad, kDbgEmabIso))
-            continue;
-        float4 c[4];
+    const int nrc = tb.rho.n - 1, nec = NE - 1, ntc = tb.t.n - 1;
+    const long long dY = (long long)ntc * nrc * nec, sp0 = (long long)species * tb.ye.n;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < p; i0 += U * step) {
+        float fr[U], ft[U], fy[U], fe[U];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) c[k] = __ldg(tab + base + (k & 1) * dT + (k >> 1) * dY);
-        const float c0 = c[0].x;
-        float v = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float wk = ((k & 1) ? tt : 1.0f - tt) * ((k >> 1) ? ty : 1.0f - ty);
-            // rho_i and rho_i+1, each linear in ln E between the two energy nodes
-            const float a0 = fmaf(te, c[k].z - c[k].x, c[k].x - c0);
-            const float a1 = fmaf(te, c[k].w - c[k].y, c[k].y - c0);
-            v = fmaf(wk, fmaf(tr, a1 - a0, a0), v);
+        for (int u = 0; u < U; ++u) {
+            const long long i = i0 + u * step < p ? i0 + u * step : i0;
+            fr[u] = narrow(rho[i]);
+            ft[u] = narrow(T[i]);
+            fy[u] = narrow(Ye[i]);
+            fe[u] = narrow(E[i]);
         }
-        out[i] = (double)expf(c0 + v);
+        float tr[U], tt[U], ty[U], te[U];
+        float4 c[U][4];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            int ir, it, iy;
+            cell_f(log10f(fr[u]), tb.rho, &ir, &tr[u]);
+            cell_f(log10f(ft[u]), tb.t, &it, &tt[u]);
+            cell_f(fy[u], tb.ye, &iy, &ty[u]);
+            float le = logf(fe[u]);
+            if (!(le >= lo_e)) le = lo_e;
+            if (le > hi_e) le = hi_e;
+            const int b = (int)((le - lo_e) * scale);
+            const int lo = cell_from(lne, NE, le, (int)lut[b < kBuckets ? b : kBuckets - 1]);
+            te[u] = (le - lne[lo]) / (lne[lo + 1] - lne[lo]);
+            // the (T, rho, E) cell's eight corners are one 32-byte sector; (T, Ye) corners k = cb + 2 cc
+            const long long base = (((sp0 + iy) * ntc + it) * nrc + ir) * nec + lo;
+            const bool ok = NMC_IN_BOUNDS(g.dbg, base, tb.n_quad, kDbgEmabIso) &&
+                            NMC_IN_BOUNDS(g.dbg, base + dY, tb.n_quad, kDbgEmabIso);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) c[u][k] = ok ? __ldg(tab + 2 * (base + (k >> 1) * dY) + (k & 1)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float c0 = c[u][0].x;
+            float v = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float wk = ((k & 1) ? tt[u] : 1.0f - tt[u]) * ((k >> 1) ? ty[u] : 1.0f - ty[u]);
+                // rho_i and rho_i+1, each linear in ln E between the two energy nodes
+                const float a0 = fmaf(te[u], c[u][k].z - c[u][k].x, c[u][k].x - c0);
+                const float a1 = fmaf(te[u], c[u][k].w - c[u][k].y, c[u][k].y - c0);
+                v = fmaf(wk, fmaf(tr[u], a1 - a0, a0), v);
+            }
+            if (i0 + u * step < p) out[i0 + u * step] = widen(expf(c0 + v));
+        }
+    }
+}
+
+// The FP32 ln table [ns][nye][nt][nrho][ne] regrouped per (T, rho, E) cell (DevTables::emab_q).
+__global__ void f32_cells_kernel(const float* __restrict__ tab, long long nsy, int nt, int nr, int ne, float4* __restrict__ out) {
+    const long long nrc = nr - 1, nec = ne - 1, ntc = nt - 1, total = nsy * ntc * nrc * nec;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const long long e = i % nec, ir = (i / nec) % nrc, it = (i / (nec * nrc)) % ntc, sy = i / (nec * nrc * ntc);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float* r0 = tab + ((sy * nt + it + k) * nr + ir) * ne + e;
+            out[2 * i + k] = make_float4(r0[0], r0[ne], r0[1], r0[ne + 1]);
+        }
     }
 }
 
 }  // namespace
+
+int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev) {
+    const DevTables& t = ctx->tb;
+    const long long nsy = (long long)ctx->ns * t.ye.n;
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, (size_t)t.n_quad * 2 * sizeof(float4));
+    if (e != cudaSuccess) return set_error(ctx, NMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    ctx->allocations.push_back(p);
+    f32_cells_kernel<<<ctx->num_sms * 8, 256>>>(tab, nsy, t.t.n, t.rho.n, ctx->ne, static_cast<float4*>(p));
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("FP32 cells: ") + cudaGetErrorString(e));
+    *dev = static_cast<const float4*>(p);
+    return NMC_OK;
+}
 
 int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     InterpTables& fx = ctx->fx;
@@ -332,6 +419,7 @@ int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("fixed-point tables: ") + cudaGetErrorString(e));
+    fx.n_quad = nrows * (tb->n_rho - 1) * (ne - 1);
     fx.quads[0] = q[0];
     fx.quads[1] = q[1];
     return NMC_OK;
@@ -340,12 +428,15 @@ int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
 int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                                 const double* T, const double* Ye, const double* E, double* out,
                                 cudaStream_t stream) {
-    const int threads = 256;
+    const int threads = kBuckets;
     long long blocks = (p + threads - 1) / threads;
     const long long cap = (long long)ctx->num_sms * 8;
-    if (blocks > cap) blocks = cap;
-    opacity_interp_mixed_kernel<<<(unsigned)blocks, threads, 0, stream>>>(ctx->g, ctx->tb, which, species, p, rho, T,
-                                                                          Ye, E, out);
+    // two points a thread once every SM has its blocks; below that one, so that the points spread over the SMs
+    if (blocks >= 2 * cap)
+        opacity_interp_mixed_kernel<2><<<(unsigned)cap, threads, 0, stream>>>(ctx->g, ctx->tb, which, species, p, rho, T, Ye, E, out);
+    else
+        opacity_interp_mixed_kernel<1><<<(unsigned)(blocks > cap ? cap : blocks), threads, 0, stream>>>(ctx->g, ctx->tb, which,
+                                                                                                  species, p, rho, T, Ye, E, out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return set_error(ctx, NMC_ECUDA, std::string("opacity_interp_mixed launch: ") + cudaGetErrorString(e));
@@ -355,7 +446,7 @@ int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long 
 int launch_opacity_interp(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                           const double* T, const double* Ye, const double* E, double* out,
                           cudaStream_t stream) {
-    const int threads = 256;
+    const int threads = kBuckets;
     long long blocks = (p + threads - 1) / threads;
     const long long cap = (long long)ctx->num_sms * 8;
     if (blocks > cap) blocks = cap;

@@ -79,3 +79,18 @@ def test_fixed_point_matches_fp64(n_elem, de1, nq, ns, n):
             assert np.sqrt(np.mean(((a - r) / r) ** 2)) <= max(1.5 * np.sqrt(np.mean(((b - r) / r) ** 2)), 1e-15)
     fixed.close()
     fp64.close()
+
+
+@pytest.mark.parametrize("n", [1, 255, 152 * 8 * 256, 152 * 16 * 256 - 1, 152 * 16 * 256 + 1, 1000003])
+def test_points_do_not_depend_on_the_batch(n):
+    """Sizes around one and two points a thread: every point's value is the one it has in a call of its own few
+    thousand neighbours, bit for bit, in both precisions (each point is evaluated by itself)."""
+    edges, g, tables, _ = make_case(10, 3.0, 2, 2, "profile", 1)
+    ctx = nmc.Context(edges, 2, 2, tables)
+    pts = [p.contiguous() for p in _points(np.random.default_rng(6), g, n)]
+    for mixed in (False, True):
+        whole = ctx.opacity_interp(1, 1, *pts, mixed=mixed)
+        for i in sorted({0, max(0, n // 2 - 1000), max(0, n - 2000)}):
+            part = ctx.opacity_interp(1, 1, *[p[i:i + 2000].contiguous() for p in pts], mixed=mixed)
+            assert torch.equal(part, whole[i:i + 2000])
+    ctx.close()
