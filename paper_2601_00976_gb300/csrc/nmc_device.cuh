@@ -52,6 +52,9 @@ __device__ __forceinline__ double abs_max(double a, double b) {
     if (kb > kInfBits) kb = 0;
     return __longlong_as_double((long long)(ka > kb ? ka : kb));
 }
+// biased exponent; normal: neither zero, denormal, infinite nor NaN
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ bool normal_exponent(int e) { return (unsigned)(e - 1) < 2046u; }
 // x <= t for x >= 0 or NaN (false) and t >= 0
 __device__ __forceinline__ bool nonneg_le(double x, double t) { return bits_of(x) <= bits_of(t); }
 __device__ __forceinline__ bool nonneg_le(float x, float t) { return x <= t; }
@@ -393,7 +396,10 @@ __device__ inline void anderson_solve(const double (&G)[MAXM][MAXM], int m, doub
 // A_ij = <F_L - F_gi, F_L - F_gj> and r_i = <F_L - F_gi, F_L> over the window
 // g0 < g1 < L of n + 1 = m columns.  Every lane gets the coefficients (c0, c1,
 // cL) of columns g0, g1 (n = 2) and L; a numerically singular system gives the
-// Picard step (0, 0, 1).
+// Picard step (0, 0, 1).  The pivot tests against 1e-14 (= 2^-46.5) dmax are decided by the exponents
+// where these suffice (|p0| >= 2^ep, dmax < 2^(ed + 1): true from ep = ed - 45 on; the determinant's
+// likewise, biased exponents), and by the products, two FP64 instructions on the solve's critical path,
+// only near the line.
 __device__ __forceinline__ void anderson3_warp(double e, int n, double& c0, double& c1, double& cL) {
     const int lane = threadIdx.x & 31;
     const double a00 = __shfl_sync(kFull, e, 0), a01 = __shfl_sync(kFull, e, 1);
@@ -414,7 +420,8 @@ __device__ __forceinline__ void anderson3_warp(double e, int n, double& c0, doub
             const bool sw = abs_gt(a01, __longlong_as_double((long long)abs_bits(a00)));
             const double p0 = sw ? a01 : a00, p1 = sw ? a11 : a01, pr = sw ? r1 : r0;
             const double q0 = sw ? a00 : a01, q1 = sw ? a01 : a11, qr = sw ? r0 : r1;
-            if (abs_gt(p0, 1e-14 * dmax)) {
+            const int ed = exponent_of(dmax), ep = exponent_of(p0);
+            if (normal_exponent(ep) && ep >= ed - 45 || abs_gt(p0, 1e-14 * dmax)) {
                 // lane 0: det = p0 q1 - q0 p1; lane 1: p0 qr - q0 pr (gamma1 det);
                 // lane 2: pr q1 - p1 qr (gamma0 det), as one x y - z w
                 const double x = lane == 2 ? pr : p0;
@@ -423,7 +430,8 @@ __device__ __forceinline__ void anderson3_warp(double e, int n, double& c0, doub
                 const double w = lane == 0 ? p1 : (lane == 1 ? pr : qr);
                 const double t = x * y - z * w;
                 const double det = __shfl_sync(kFull, t, 0);
-                if (abs_gt(det, 1e-14 * dmax * fabs(p0))) {
+                const int et = exponent_of(det);
+                if (normal_exponent(et) && et >= ed + ep - 1067 || abs_gt(det, 1e-14 * dmax * fabs(p0))) {
                     const double gm = t * (1.0 / det);
                     const double gm1 = __shfl_sync(kFull, gm, 1), gm0 = __shfl_sync(kFull, gm, 2);
                     const double sum = gm0 + gm1;
@@ -574,6 +582,7 @@ struct OpacBufs {
 //    q >= q' and completed by detailed balance, K_Out[q'][q] = a_q / a_q'
 //    K_Out[q][q'] for q' < q (Eqs. inOutInvarianceNES, detailedBalanceNES),
 //    and the pair kernel K_Ann of each particle/antiparticle pair.
+// mu_T: (T, Ye, mu_e) of an EoS evaluation at this rho, or null; spares the root (FP64) at that state.
 // The warp of thread `lead` (lane 0 of its warp) does the scalar part; `lead`
 // ORs NMC_TABLE_CLAMP into *status when a lookup leaves a table.
 // Ends with the block synchronised.
@@ -588,7 +597,8 @@ constexpr int kFillBatchF64 = 4;
 template <typename R>
 __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const nmc_params& P, double rho, double T,
                                   double Ye, double dtau, const double* sc, const OpacBufs<R>& b, OpacState* os,
-                                  int* status, R& chiab, R& sig, R& deq, R& deqc, int lead = 0) {
+                                  int* status, R& chiab, R& sig, R& deq, R& deqc, int lead = 0,
+                                  const double* mu_T = nullptr) {
     constexpr bool kMixed = sizeof(R) == 4;
     const int NS = g.ns, NE = g.ne, NEP = g.nep, LD = g.ld;
     const int GS = NEP;   // threads per species
@@ -610,9 +620,16 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
         // mixed: the FP32 root of the electron cubic, then one FP64 Newton step on it (the error
         // squares): mu_e, and with it D^Eq, must move smoothly with (T, Ye), or the outer
         // iteration's map is noisy at the 1e-7 level and stalls above tol_outer
-        const double mu_e = kMixed ? eos_mu_e_refined(rho, T, Ye) : eos_mu_e(rho, T, Ye);
+        double tinv, mu_e;
+        if constexpr (kMixed) {
+            mu_e = eos_mu_e_refined_warp(rho, T, Ye, &tinv);
+        } else if (mu_T && bits_of(mu_T[0]) == bits_of(T) && bits_of(mu_T[1]) == bits_of(Ye)) {
+            mu_e = mu_T[2];   // the EoS was last evaluated at this very state
+            tinv = 1.0 / T;
+        } else {
+            mu_e = eos_mu_e_warp(Ye * rho / kMB, T, &tinv);
+        }
         const double mnu = mu_e - (T * lratio + kDmNP);   // mu_e - mu_hat
-        const double tinv = 1.0 / T;
         const double eta_e = mu_e / T;
         // table cells in FP64 in both precisions, lane 0: log10 rho, 1: log10 T (EmAb/Iso axis),
         // 2: Ye, 3: log10 T (kernel axis), 4: eta_e
@@ -728,8 +745,13 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
         // the quadrature points taken in order, their operator weights loaded kProjQuad / 2 points at a
         // time.  With D^Eq also a = D^Eq / (1 - D^Eq) and 1 / a, which the detailed-balance fill of the
         // NES kernel reads across the species.
+        // The ns n_elem tasks are dealt out to consecutive threads from the lead warp on: one full warp
+        // instead of several partly empty ones (an instruction costs the same), on SMSPs that change
+        // with the node.
         constexpr int kHalfQ = kProjQuad / 2;
-        for (int e = q; s < NS && e < g.n_elem; e += GS) {
+        const int task0 = tid >= lead ? tid - lead : tid - lead + (int)blockDim.x;
+        for (int task = task0; task < NS * g.n_elem; task += blockDim.x) {
+            const int s = task / g.n_elem, e = task - s * g.n_elem;
             const int nq = g.nq;
             if (!NMC_IN_BOUNDS(g.dbg, ((long long)e * nq + nq - 1) * kProjQuad + kProjQuad - 1,
                                (long long)g.n_elem * nq * kProjQuad, kDbgProj) ||

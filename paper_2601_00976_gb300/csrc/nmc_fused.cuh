@@ -67,8 +67,10 @@ template <int MAXM>
 struct NodeShared {
     double rho, dtau, T;
     double sc[4];
-    double y[2], ystar[2], qv[2];
+    double y[2], ystar[2];
     double k_eps, k_ye, ri_ys[2];
+    double nb, ku;                // rho / m_B, (MeV in erg) / ((hbar c)^3 rho)
+    double mu_T[3];               // T, Ye, mu_e of the last EoS evaluation (FP64 path)
     double EN_star[2];
     double qh[kMaxOuterMem][2], fh[kMaxOuterMem][2];
     double G[MAXM][MAXM];
@@ -179,31 +181,45 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
             Isd[1] = a.H[o * 3 + 1];
             Isd[2] = a.H[o * 3 + 2];
         }
-        if (tid == lead) {
+        if ((tid >> 5) == (lead >> 5)) {   // the lead warp, every lane carrying the node's scalars
+            const int ln = tid & 31;
             const double rho = a.rho[n], T = a.T[n], Ye = a.Ye[n], dt = a.dt[n];
-            nd->rho = rho;
-            nd->T = T;
-            nd->dtau = kC * dt;
-            for (int k = 0; k < 4; ++k) nd->sc[k] = a.scale ? a.scale[n * 4 + k] : 1.0;
             const bool okin = rho > 0.0 && isfinite(rho) && T > 0.0 && isfinite(T) &&
                               Ye > 0.0 && Ye < 1.0 && dt >= 0.0 && isfinite(dt);
-            nd->status = okin ? 0 : NMC_BAD_INPUT;
-            double e = 0.0, de = 0.0;
-            if (okin) eos_eps(rho, T, Ye, &e, &de);
-            nd->ystar[0] = e;
-            nd->ystar[1] = Ye;
-            // per-node factors of the matter update: eps and Ye per unit change of the neutrino
-            // energy and lepton number densities, and the outer residuals' scales 1 / |y*|
-            nd->k_eps = kMeVErg / rho;
-            nd->k_ye = kMB / rho;
-            nd->ri_ys[0] = 1.0 / fabs(e);
-            nd->ri_ys[1] = 1.0 / fabs(Ye);
-            nd->y[0] = e;
-            nd->y[1] = Ye;
-            nd->n_inner = 0;
-            nd->n_outer = 0;
-            nd->bad = 0;
-            nd->done = okin ? 0 : 1;
+            // per-node factors, one division on different lanes: rho / m_B, n_e, and those of the matter
+            // update (eps and Ye per unit change of the neutrino energy and lepton number densities)
+            const double d = (ln == 0 ? rho : (ln == 1 ? Ye * rho : (ln == 2 ? kMB : kMeVErg))) /
+                             (ln < 2 ? kMB : (ln == 4 ? kHbarC * kHbarC * kHbarC * rho : rho));
+            const double nb = lane_value(d, 0), k_eps = lane_value(d, 3);
+            double e = 0.0, de = 0.0, mu = 0.0;
+            if (okin) {
+                mu = eos_mu_e_warp(lane_value(d, 1), T);
+                eos_eps_at_mu_warp(nb, k_eps, T, mu, &e, &de);
+            }
+            const double ri = 1.0 / fabs(ln == 0 ? e : Ye);   // the outer residuals' scales 1 / |y*|
+            if (ln < 2) nd->ri_ys[ln] = ri;
+            if (ln < 4) nd->sc[ln] = a.scale ? a.scale[n * 4 + ln] : 1.0;
+            if (ln == 2) nd->k_ye = d;
+            if (ln == 4) nd->ku = d;
+            if (ln == 0) {
+                nd->rho = rho;
+                nd->T = T;
+                nd->dtau = kC * dt;
+                nd->nb = nb;
+                nd->k_eps = k_eps;
+                nd->mu_T[0] = T;
+                nd->mu_T[1] = Ye;
+                nd->mu_T[2] = mu;
+                nd->status = okin ? 0 : NMC_BAD_INPUT;
+                nd->ystar[0] = e;
+                nd->ystar[1] = Ye;
+                nd->y[0] = e;
+                nd->y[1] = Ye;
+                nd->n_inner = 0;
+                nd->n_outer = 0;
+                nd->bad = 0;
+                nd->done = okin ? 0 : 1;
+            }
         }
         __syncthreads();
         if (nd->done) {   // invalid input: outputs = inputs
@@ -244,7 +260,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
             // D^Eq of the first outer iteration stay in place (nothing else writes them)
             if (k == 1 || !P.semi_implicit)
                 compute_opacities<R>(g, a.tb, P, nd->rho, nd->T, nd->y[1], nd->dtau, nd->sc, ob, &nd->op,
-                                     &nd->status, chiab, sig, deq, deqc, lead);
+                                     &nd->status, chiab, sig, deq, deqc, lead, nd->mu_T);
             NMC_TRACE_TICK(kTrOpac);
             if constexpr (kMixed) {
                 const double c1 = (double)Wt, c2 = c1 * (double)chiab;
@@ -508,14 +524,14 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                         if (k < K)
                             for (int i = 0; i < (int)(blockDim.x >> 5); ++i) sk += pr[i * K + k];
                         double e;
-                        if constexpr (kMixed) e = (double)sk;
+                        if constexpr (kMixed) e = widen(sk);
                         else e = gram3_update_warp<3>(nd->G, sk, m);
                         double c0, c1, cL;
                         anderson3_warp(e, m - 1, c0, c1, cL);
                         if (k < 3) {
                             const double a = anderson3_coef(k, m - 1, c0, c1, cL);
-                            nd->alpha[k] = a;
-                            nd->alpha_f[k] = (float)a;
+                            if constexpr (kMixed) nd->alpha_f[k] = narrow(a);
+                            else nd->alpha[k] = a;
                         }
                     }
                     __syncthreads();
@@ -622,20 +638,21 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                     const double qv0 = nd->ystar[0] - (nd->blk_out[0] - nd->EN_star[0]) * nd->k_eps;
                     const double qv1 = nd->ystar[1] - (nd->blk_out[1] - nd->EN_star[1]) * nd->k_ye;
                     const double y0 = nd->y[0], y1 = nd->y[1];
-                    if (ln == 0) { nd->qv[0] = qv0; nd->qv[1] = qv1; }
                     const int mo = k < P.m_outer ? k : P.m_outer;
                     double yn0, yn1;
                     outer_step_warp(nd->qh, nd->fh, qv0, qv1, y0, y1, nd->ri_ys, mo, yn0, yn1);
-                    const int conv = fabs(yn0 - y0) <= P.tol_outer * fabs(nd->ystar[0]) &&
-                                     fabs(yn1 - y1) <= P.tol_outer * fabs(nd->ystar[1]);   // Algorithm 3
+                    const int conv = nonneg_le(fabs(yn0 - y0), P.tol_outer * fabs(nd->ystar[0])) &&
+                                     nonneg_le(fabs(yn1 - y1), P.tol_outer * fabs(nd->ystar[1]));   // Algorithm 3
                     int stop = conv, st = 0;
                     double Tn = nd->T;
                     if (!(is_finite(yn0) && is_finite(yn1))) { st |= NMC_NONFINITE; stop = 1; }
                     if (!stop && k >= P.max_outer) { st |= NMC_NOT_CONVERGED_OUTER; stop = 1; }
                     if (!stop) {   // an iterate outside the EoS domain stops the node
                         bool ok;
-                        const double Tk = kMixed ? eos_temperature_mixed(rho, yn0, yn1, Tn, &ok)
-                                                 : eos_temperature(rho, yn0, yn1, Tn, &ok);
+                        double mu_T[3] = {0.0, 0.0, 0.0};
+                        const double Tk = kMixed ? eos_temperature_mixed_warp(rho, nd->nb, nd->k_eps, nd->ku, yn0, yn1, Tn, &ok)
+                                                 : eos_temperature_warp(rho, nd->nb, nd->k_eps, yn0, yn1, Tn, &ok, mu_T);
+                        if (!kMixed && ln < 3) nd->mu_T[ln] = ln == 0 ? mu_T[0] : (ln == 1 ? mu_T[1] : mu_T[2]);
                         if (ok) Tn = Tk;
                         else { st |= NMC_EOS_FAIL; stop = 1; }
                     }
@@ -661,32 +678,33 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
             const double Dcur = kMixed ? f2_to(Dx) : (double)M[0];
             double v[2] = {W3q * Dcur, gs * W2q * Dcur};
             block_sum<2, double>(v, red, nd->blk_out);
-            if (tid == lead) {
-                nd->qv[0] = nd->ystar[0] - (nd->blk_out[0] - nd->EN_star[0]) * nd->k_eps;
-                nd->qv[1] = nd->ystar[1] - (nd->blk_out[1] - nd->EN_star[1]) * nd->k_ye;
-            }
         }
-        if (tid == lead) {
+        if ((tid >> 5) == (lead >> 5)) {
             const double rho = nd->rho;
+            const double qv0 = nd->ystar[0] - (nd->blk_out[0] - nd->EN_star[0]) * nd->k_eps;
+            const double qv1 = nd->ystar[1] - (nd->blk_out[1] - nd->EN_star[1]) * nd->k_ye;
+            int st = nd->status;
             double yo0, yo1, To;
             if (P.frozen_matter) {
                 yo0 = nd->ystar[0]; yo1 = nd->ystar[1]; To = a.T[n];
-            } else if (nd->status & NMC_NONFINITE) {
+            } else if (st & NMC_NONFINITE) {
                 yo0 = nd->y[0]; yo1 = nd->y[1]; To = nd->T;
             } else {
-                if (P.final_q) { yo0 = nd->qv[0]; yo1 = nd->qv[1]; }   // y = q(M, y) at converged M
-                else { yo0 = nd->y[0]; yo1 = nd->y[1]; }                // Anderson-mixed iterate
+                if (P.final_q) { yo0 = qv0; yo1 = qv1; }   // y = q(M, y) at converged M
+                else { yo0 = nd->y[0]; yo1 = nd->y[1]; }    // Anderson-mixed iterate
                 bool ok;
-                To = kMixed ? eos_temperature_mixed(rho, yo0, yo1, nd->T, &ok)
-                            : eos_temperature(rho, yo0, yo1, nd->T, &ok);
-                if (!ok) { nd->status |= NMC_EOS_FAIL; To = nd->T; }   // last T inside the domain
+                To = kMixed ? eos_temperature_mixed_warp(rho, nd->nb, nd->k_eps, nd->ku, yo0, yo1, nd->T, &ok)
+                            : eos_temperature_warp(rho, nd->nb, nd->k_eps, yo0, yo1, nd->T, &ok, nullptr);
+                if (!ok) { st |= NMC_EOS_FAIL; To = nd->T; }   // last T inside the domain
             }
-            a.Ye_out[n] = yo1;
-            a.eps_out[n] = yo0;
-            a.T_out[n] = To;
-            a.n_outer[n] = nd->n_outer;
-            a.n_inner[n] = nd->n_inner;
-            a.status[n] = (uint32_t)nd->status;
+            if (tid == lead) {
+                a.Ye_out[n] = yo1;
+                a.eps_out[n] = yo0;
+                a.T_out[n] = To;
+                a.n_outer[n] = nd->n_outer;
+                a.n_inner[n] = nd->n_inner;
+                a.status[n] = (uint32_t)st;
+            }
         }
         if (act && NMC_IN_BOUNDS(g.dbg, (n * NS + s) * NE + q, a.n * NS * NE, kDbgOutput)) {
             const long long o = (n * NS + s) * NE + q;

@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "nmc_internal.h"
+#include "nmc_eos.cuh"
 
 namespace nmc {
 
@@ -249,23 +250,6 @@ int upload_fx(nmc_ctx* ctx, const T* host, size_t count, const T** dev) {
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));
     *dev = static_cast<const T*>(p);
     return NMC_OK;
-}
-
-// (float)x and (double)x in integers, the same values bit for bit: a conversion instruction runs on the FP64
-// pipe (~64 cycles of an SMSP), and a point of the FP32 form needs five.  Values whose FP32 form is not a
-// normal number take the instruction.
-__device__ __forceinline__ float narrow(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x);
-    if (((hi >> 20) & 0x7ffu) - 897u > 253u) return (float)x;
-    const uint64_t u = word_of(x);
-    const uint64_t t = u + 0x0fffffffull + ((u >> 29) & 1u);   // round to nearest, ties to even
-    return __uint_as_float(((unsigned)(t >> 29) - (896u << 23)) | (hi & 0x80000000u));
-}
-
-__device__ __forceinline__ double widen(float x) {
-    const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
-    if (e - 1u > 253u) return (double)x;
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
 }
 
 __device__ __forceinline__ void cell_f(float v, const Axis& ax, int* i, float* t) {

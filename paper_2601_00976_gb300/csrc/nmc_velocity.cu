@@ -52,6 +52,7 @@ struct VelNode {
     double y[kNy], ystar[kNy], ri[kNy];   // matter iterate, old state, 1 / Algorithm 3 reference
     double Fs[3], Es, Ns;                 // Eulerian momentum, energy and number of the old state
     double cf, k_eps, k_ye, lam;          // MeV/(rho c^2), MeV/rho, m_B/rho, 1/(1+|v|)
+    double nb, mu_T[3];                   // rho / m_B; T, Ye, mu_e of the last EoS evaluation
     double qh[kMaxOuterMem][kNy], fh[kMaxOuterMem][kNy];
     double G[3][3];
     double alpha[3];
@@ -226,34 +227,58 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
             for (int j = 0; j < 3; ++j) Is[j] = a.H[o * 3 + j];
         }
         const double vs[3] = {va.v_in[n * 3 + 0], va.v_in[n * 3 + 1], va.v_in[n * 3 + 2]};
-        if (tid == lead) {
+        if ((tid >> 5) == (lead >> 5)) {   // the lead warp, every lane carrying the node's scalars
+            const int ln = tid & 31;
             const double rho = a.rho[n], T = a.T[n], Ye = a.Ye[n], dt = a.dt[n];
             const double v2 = vs[0] * vs[0] + vs[1] * vs[1] + vs[2] * vs[2];
             const bool okin = rho > 0.0 && isfinite(rho) && T > 0.0 && isfinite(T) && Ye > 0.0 && Ye < 1.0 &&
                               dt >= 0.0 && isfinite(dt) && v2 < 1.0;   // v2 < 1 also rejects NaN
-            nd->rho = rho;
-            nd->T = T;
-            nd->dtau = kC * dt;
-            for (int k = 0; k < 4; ++k) nd->sc[k] = a.scale ? a.scale[n * 4 + k] : 1.0;
-            nd->status = okin ? 0 : NMC_BAD_INPUT;
-            double e = 0.0, de = 0.0;
-            if (okin) eos_eps(rho, T, Ye, &e, &de);
             const double c2 = kC * kC;
-            for (int j = 0; j < 3; ++j) nd->ystar[j] = nd->y[j] = vs[j];
-            nd->ystar[3] = nd->y[3] = e + 0.5 * v2 * c2;
-            nd->ystar[4] = nd->y[4] = Ye;
-            const double vref = fmax(sqrt(v2), va.v_floor);
-            nd->ri[0] = nd->ri[1] = nd->ri[2] = 1.0 / vref;
-            nd->ri[3] = 1.0 / fabs(nd->ystar[3]);
-            nd->ri[4] = 1.0 / fabs(Ye);
-            nd->cf = kMeVErg / (rho * c2);
-            nd->k_eps = kMeVErg / rho;
-            nd->k_ye = kMB / rho;
-            nd->lam = 1.0 / (1.0 + sqrt(v2));
-            nd->n_inner = 0;
-            nd->n_outer = 0;
-            nd->bad = 0;
-            nd->done = okin ? 0 : 1;
+            const double sv = sqrt(v2);
+            // per-node factors, one division on different lanes
+            double num = kMeVErg, den = rho;                      // lane 0: MeV / rho
+            if (ln == 1) num = kMB;                               // m_B / rho
+            if (ln == 2) den = rho * c2;                          // MeV / (rho c^2)
+            if (ln == 3) { num = rho; den = kMB; }                // rho / m_B
+            if (ln == 4) { num = Ye * rho; den = kMB; }           // n_e
+            if (ln == 5) { num = 1.0; den = 1.0 + sv; }           // lambda
+            if (ln == 6) { num = 1.0; den = fmax(sv, va.v_floor); }
+            if (ln == 7) { num = 1.0; den = fabs(Ye); }
+            const double d = num / den;
+            const double nb = lane_value(d, 3), k_eps = lane_value(d, 0);
+            double e = 0.0, de = 0.0, mu = 0.0;
+            if (okin) {
+                mu = eos_mu_e_warp(lane_value(d, 4), T);
+                eos_eps_at_mu_warp(nb, k_eps, T, mu, &e, &de);
+            }
+            const double ef = e + 0.5 * v2 * c2;
+            const double rv = lane_value(d, 6), rYe = lane_value(d, 7), lam = lane_value(d, 5), cf = lane_value(d, 2);
+            const double k_ye = lane_value(d, 1);
+            if (ln < 4) nd->sc[ln] = a.scale ? a.scale[n * 4 + ln] : 1.0;
+            if (ln == 0) {
+                nd->rho = rho;
+                nd->T = T;
+                nd->dtau = kC * dt;
+                nd->nb = nb;
+                nd->status = okin ? 0 : NMC_BAD_INPUT;
+                for (int j = 0; j < 3; ++j) nd->ystar[j] = nd->y[j] = vs[j];
+                nd->ystar[3] = nd->y[3] = ef;
+                nd->ystar[4] = nd->y[4] = Ye;
+                nd->ri[0] = nd->ri[1] = nd->ri[2] = rv;
+                nd->ri[3] = 1.0 / fabs(ef);
+                nd->ri[4] = rYe;
+                nd->cf = cf;
+                nd->k_eps = k_eps;
+                nd->k_ye = k_ye;
+                nd->lam = lam;
+                nd->mu_T[0] = T;
+                nd->mu_T[1] = Ye;
+                nd->mu_T[2] = mu;
+                nd->n_inner = 0;
+                nd->n_outer = 0;
+                nd->bad = 0;
+                nd->done = okin ? 0 : 1;
+            }
         }
         __syncthreads();
         if (nd->done) {   // invalid input: outputs = inputs
@@ -302,7 +327,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
             // and this thread's chiab, sig and D^Eq stay in place for the later outer iterations
             if (k == 1 || !P.semi_implicit)
                 compute_opacities<double>(g, a.tb, P, nd->rho, nd->T, nd->y[4], nd->dtau, nd->sc, ob, &nd->op,
-                                          &nd->status, chiab, sig, deq, deqc, lead);
+                                          &nd->status, chiab, sig, deq, deqc, lead, nd->mu_T);
             const double vk[3] = {nd->y[0], nd->y[1], nd->y[2]};
             const double lam = nd->lam;
             {   // reference norm ||D^[k,1]||_W per species and the Algorithm 2 thresholds
@@ -495,7 +520,10 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                     if (!stop && k >= P.max_outer) { st |= NMC_NOT_CONVERGED_OUTER; stop = 1; }
                     if (!stop) {   // an iterate outside the EoS domain stops the node
                         bool ok;
-                        const double Tk = eos_temperature(rho, yn[3] - 0.5 * vn2 * kC * kC, yn[4], Tn, &ok);
+                        double mu_T[3] = {0.0, 0.0, 0.0};
+                        const double Tk = eos_temperature_warp(rho, nd->nb, nd->k_eps, yn[3] - 0.5 * vn2 * kC * kC, yn[4], Tn,
+                                                               &ok, mu_T);
+                        if (ln < 3) nd->mu_T[ln] = ln == 0 ? mu_T[0] : (ln == 1 ? mu_T[1] : mu_T[2]);
                         if (ok) Tn = Tk;
                         else { st |= NMC_EOS_FAIL; stop = 1; }
                     }
@@ -521,14 +549,15 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
             eulerian_terms(M[0], &M[1], W3q, gs * W2q, t);
             block_sum<kNsum, double>(t, red, nd->blk_out);
         }
-        if (tid == lead) {
+        if ((tid >> 5) == (lead >> 5)) {
             const double rho = nd->rho;
+            int st = nd->status;
             const double* S = nd->blk_out;
             double v[3] = {nd->ystar[0], nd->ystar[1], nd->ystar[2]};
             double eps_f = nd->ystar[3], Ye = nd->ystar[4], To = a.T[n];
             if (P.frozen_matter) {
                 // y = y*
-            } else if (nd->status & NMC_NONFINITE) {
+            } else if (st & NMC_NONFINITE) {
                 for (int j = 0; j < 3; ++j) v[j] = nd->y[j];
                 eps_f = nd->y[3];
                 Ye = nd->y[4];
@@ -566,17 +595,19 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                 }
                 bool ok;
                 const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-                To = eos_temperature(rho, eps_f - 0.5 * v2 * kC * kC, Ye, nd->T, &ok);
-                if (!ok) { nd->status |= NMC_EOS_FAIL; To = nd->T; }
+                To = eos_temperature_warp(rho, nd->nb, nd->k_eps, eps_f - 0.5 * v2 * kC * kC, Ye, nd->T, &ok, nullptr);
+                if (!ok) { st |= NMC_EOS_FAIL; To = nd->T; }
             }
             const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-            for (int j = 0; j < 3; ++j) va.v_out[n * 3 + j] = v[j];
-            a.Ye_out[n] = Ye;
-            a.eps_out[n] = eps_f - 0.5 * v2 * kC * kC;
-            a.T_out[n] = To;
-            a.n_outer[n] = nd->n_outer;
-            a.n_inner[n] = nd->n_inner;
-            a.status[n] = (uint32_t)nd->status;
+            if (tid == lead) {
+                for (int j = 0; j < 3; ++j) va.v_out[n * 3 + j] = v[j];
+                a.Ye_out[n] = Ye;
+                a.eps_out[n] = eps_f - 0.5 * v2 * kC * kC;
+                a.T_out[n] = To;
+                a.n_outer[n] = nd->n_outer;
+                a.n_inner[n] = nd->n_inner;
+                a.status[n] = (uint32_t)st;
+            }
         }
         if (act) {
             const long long o = (n * NS + s) * NE + q;
