@@ -40,6 +40,7 @@ __device__ __forceinline__ unsigned long long bits_of(double x) { return (unsign
 __device__ __forceinline__ unsigned long long abs_bits(double x) { return bits_of(x) & 0x7fffffffffffffffull; }
 __device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x7ff00000; }
 __device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool is_positive(double x) { return bits_of(x) - 1 < kInfBits; }   // x > 0 (NaN: no)
 // |a| > b for b >= 0 (false when either is NaN)
 __device__ __forceinline__ bool abs_gt(double a, double b) {
     const unsigned long long ka = abs_bits(a);
