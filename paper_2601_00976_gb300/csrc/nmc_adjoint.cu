@@ -58,6 +58,7 @@ namespace {
 
 struct AdjNode {
     double rho, dtau, T, Tp;
+    double nb, f;            // rho / m_B, (MeV in erg) / rho
     double Tq[4], yq[4][2];  // the four perturbed matter states of B's differences and their temperatures
     double sc[4];
     double unit[4];
@@ -66,8 +67,8 @@ struct AdjNode {
     double g_y[2];           // cotangent of y = (eps, Ye): direct, through T_out and through kappa
     double blk_out[8];
     double dinv[128];        // reciprocals of the eliminated diagonal (2 ne <= 128)
-    double cv[2][8];         // per warp: largest |entry| of the next column among its active rows,
-    double cip[2][8];        //   its reciprocal,
+    long long cv[2][8];      // per warp: bits of the largest |entry| of the next column among its active rows
+    double cip[2][8];        //   (-1: none), its reciprocal,
     int ci[2][8];            //   and its row (double-buffered by column parity)
     int prow[128];           // pivot row of each eliminated column
     OpacState op;
@@ -144,6 +145,13 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
     const bool frozen = P.frozen_matter != 0;
 
     for (long long n = blockIdx.x; n < a.n; n += gridDim.x) {
+        // The node's scalar FP64 work (the EoS solves, ComputeOpacities' scalars, a third of an SMSP's share
+        // of the node) goes to one warp.  Warp w of every resident block sits on the same SMSP, so this lead
+        // warp rotates with the node; the shift keeps blocks one SM count (a multiple of the warps) apart,
+        // which share an SM, on different SMSPs.  With the pivot search in integers (its compares were a
+        // seventh of the kernel's FP64 instructions) and the EoS on all the warp's lanes: 4099 nodes 12.7 ->
+        // 10.8 ms.
+        const int lead = (int)((n + (n >> 3)) % nwarps) << 5;
         // ---------------- inputs, y* and the output matter state ----------------
         double Ds = 0.0, D = 0.0, gD = 0.0, gIs = 0.0;   // gIs = gH . I*
         double gH[3] = {0.0, 0.0, 0.0};
@@ -159,38 +167,50 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                 }
             }
         }
-        if (tid == 0) {
+        if (warp == lead >> 5) {   // the lead warp, every lane carrying the node's scalars
             const double rho = a.rho[n], T = a.T[n], Ye = a.Ye[n], dt = a.dt[n];
-            nd->rho = rho;
-            nd->dtau = kC * dt;
-            for (int k = 0; k < 4; ++k) {
-                nd->sc[k] = a.scale ? a.scale[n * 4 + k] : 1.0;
-                nd->unit[k] = 1.0;
-            }
             const bool okin = rho > 0.0 && isfinite(rho) && T > 0.0 && isfinite(T) && Ye > 0.0 && Ye < 1.0 &&
                               dt >= 0.0 && isfinite(dt);
-            nd->status = okin ? 0 : NMC_BAD_INPUT;
-            nd->bad = okin ? 0 : 1;
-            double e = 0.0, de = 0.0;
-            if (okin) eos_eps(rho, T, Ye, &e, &de);
-            nd->ystar[0] = e;
-            nd->ystar[1] = Ye;
-            nd->deps_dT_star = de;
-            nd->deps_dYe_star = okin ? eos_deps_dye(rho, T, Ye) : 0.0;
+            // rho / m_B, n_e and (MeV in erg) / rho: one division on different lanes
+            const double d = (lane == 0 ? rho : (lane == 1 ? Ye * rho : kMeVErg)) / (lane < 2 ? kMB : rho);
+            const double nb = lane_value(d, 0), f = lane_value(d, 2);
+            double e = 0.0, de = 0.0, mu = 0.0;
+            if (okin) {
+                mu = eos_mu_e_warp(lane_value(d, 1), T);
+                eos_eps_at_mu_warp(nb, f, T, mu, &e, &de);
+            }
+            const double dy = okin ? eos_deps_dye_at_mu(T, mu) : 0.0;
+            if (lane < 4) {
+                nd->sc[lane] = a.scale ? a.scale[n * 4 + lane] : 1.0;
+                nd->unit[lane] = 1.0;
+            }
+            if (lane == 0) {
+                nd->rho = rho;
+                nd->nb = nb;
+                nd->f = f;
+                nd->dtau = kC * dt;
+                nd->status = okin ? 0 : NMC_BAD_INPUT;
+                nd->bad = okin ? 0 : 1;
+                nd->ystar[0] = e;
+                nd->ystar[1] = Ye;
+                nd->deps_dT_star = de;
+                nd->deps_dYe_star = dy;
+            }
         }
         {   // E_nu, N_nu at D* and D (Eqs. eulerianEnergyLG, eulerianNumberLG at v = 0)
             double v[4] = {W3q * Ds, gs * W2q * Ds, W3q * D, gs * W2q * D};
             block_sum<4, double>(v, red, nd->blk_out);
         }
-        if (tid == 0 && !nd->bad && !(isfinite(nd->blk_out[2]) && isfinite(nd->blk_out[3]))) {
+        if (tid == lead && !nd->bad && !(isfinite(nd->blk_out[2]) && isfinite(nd->blk_out[3]))) {
             nd->status |= NMC_NONFINITE;   // non-finite converged moments
             nd->bad = 1;
         }
-        if (tid < 32 && !nd->bad) {
-            // Warp 0: the matter state y = q(D) and the five EoS temperature solves, at y (lane 0) and at
+        __syncwarp();
+        if (warp == lead >> 5 && !nd->bad) {
+            // The lead warp: the matter state y = q(D) and the five EoS temperature solves, at y (lane 0) and at
             // the four states of B's central differences (lanes 1..4: eps + h, eps - h, Ye + h, Ye - h),
             // side by side: each solve is a chain of dependent FP64 steps, so five lanes cost one.
-            const int ln = tid;
+            const int ln = lane;
             const double rho = nd->rho;
             double y0, y1;
             if (frozen) { y0 = nd->ystar[0]; y1 = nd->ystar[1]; }
@@ -214,18 +234,20 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                 nd->yq[ln - 1][0] = yy0;
                 nd->yq[ln - 1][1] = yy1;
             }
+            // chain rule through T_out = T(eps, Ye)
+            Tk = lane_value(Tk, 0);
+            const double mu = eos_mu_e_warp(y1 * rho / kMB, Tk);
+            double e, de;
+            eos_eps_at_mu_warp(nd->nb, nd->f, Tk, mu, &e, &de);
             if (ln == 0) {
                 nd->y[0] = y0;
                 nd->y[1] = y1;
                 if (fail) { nd->status |= NMC_EOS_FAIL; nd->bad = 1; }
                 nd->T = Tk;
-                // chain rule through T_out = T(eps, Ye)
-                double e, de;
-                eos_eps(rho, Tk, y1, &e, &de);
                 const double gT = a.gT ? a.gT[n] : 0.0;
                 const double ge = a.geps ? a.geps[n] : 0.0, gy = a.gYe ? a.gYe[n] : 0.0;
                 nd->g_y[0] = ge + gT / de;
-                nd->g_y[1] = gy - gT * eos_deps_dye(rho, Tk, y1) / de;
+                nd->g_y[1] = gy - gT * eos_deps_dye_at_mu(Tk, mu) / de;
                 nd->h[0] = h0;
                 nd->h[1] = h1;
                 if (!(isfinite(nd->g_y[0]) && isfinite(nd->g_y[1]))) { nd->status |= NMC_NONFINITE; nd->bad = 1; }
@@ -242,7 +264,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
             double Qp[4] = {0.0, 0.0, 0.0, 0.0}, Kp[4] = {0.0, 0.0, 0.0, 0.0};
             for (int pass = 0; pass < 5; ++pass) {
                 // passes 0..3: (eps + h, eps - h, Ye + h, Ye - h); pass 4: unperturbed
-                if (tid == 0) {   // the pass's state, solved above
+                if (tid == lead) {   // the pass's state, solved above
                     nd->Tp = pass < 4 ? nd->Tq[pass] : nd->T;
                     nd->yp[0] = pass < 4 ? nd->yq[pass][0] : nd->y[0];
                     nd->yp[1] = pass < 4 ? nd->yq[pass][1] : nd->y[1];
@@ -251,7 +273,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                 if (nd->bad) break;
                 double chiab = 0.0, sig = 0.0, deq = 0.0, deqc = 0.0;
                 compute_opacities<double>(g, a.tb, P, nd->rho, nd->Tp, nd->yp[1], nd->dtau, nd->unit, ob, &nd->op,
-                                          &nd->status, chiab, sig, deq, deqc);
+                                          &nd->status, chiab, sig, deq, deqc, lead);
                 if (act) vAW1D[sq] = vA[sq] * Wt * (1.0 - D);
                 __syncthreads();
                 double nin = 0.0, nout = 0.0, pro = 0.0, an = 0.0;
@@ -282,7 +304,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                 {
                     double v[2] = {gk * (Kp[0] - Kp[1]) / (2.0 * nd->h[0]), gk * (Kp[2] - Kp[3]) / (2.0 * nd->h[1])};
                     block_sum<2, double>(v, red, nd->blk_out);
-                    if (tid == 0) { nd->g_y[0] += nd->blk_out[0]; nd->g_y[1] += nd->blk_out[1]; }
+                    if (tid == lead) { nd->g_y[0] += nd->blk_out[0]; nd->g_y[1] += nd->blk_out[1]; }
                 }
                 if (act) vDeq[sq] = gk;   // D^Eq is in registers by now; the slot carries g_kappa
                 __syncthreads();
@@ -350,13 +372,14 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                         return ((r < 64 ? done0 >> r : done1 >> (r - 64)) & 1ull) != 0ull;
                     };
                     if (lane == 0) {   // column 0's candidates
-                        double nb = -1.0, nip = 0.0;
+                        double nip = 0.0;
+                        long long nb = -1;
                         int ni = 0;
                         for (int r = warp; r < N2; r += nwarps) {
-                            const double v = fabs(Mt[r * LDM]);
-                            if (v > nb) { nb = v; ni = r; }
+                            const long long v = (long long)abs_bits(Mt[r * LDM]);
+                            if (v > nb && v <= (long long)kInfBits) { nb = v; ni = r; }
                         }
-                        if (nb > 0.0) nip = 1.0 / Mt[ni * LDM];
+                        if (nb > 0) nip = 1.0 / Mt[ni * LDM];
                         nd->cv[0][warp] = nb;
                         nd->ci[0][warp] = ni;
                         nd->cip[0][warp] = nip;
@@ -364,20 +387,21 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                     __syncthreads();
                     for (int c = 0; c < N2; ++c) {
                         const int bsel = c & 1;
-                        double best = -1.0, ip = 0.0;
+                        double ip = 0.0;
+                        long long best = -1;
                         int P = 0;
                         for (int w = 0; w < nwarps; ++w) {
-                            const double v = nd->cv[bsel][w];
+                            const long long v = nd->cv[bsel][w];
                             const int i = nd->ci[bsel][w];
                             if (v > best || (v == best && i < P)) { best = v; P = i; ip = nd->cip[bsel][w]; }
                         }
-                        if (!(best > 1e-300) || !isfinite(best)) {   // singular: same decision in every thread
-                            if (tid == 0) { nd->status |= NMC_NONFINITE; nd->bad = 1; }
+                        if (best <= (long long)bits_of(1e-300) || best >= (long long)kInfBits) {   // singular: same decision in every thread
+                            if (tid == lead) { nd->status |= NMC_NONFINITE; nd->bad = 1; }
                             break;
                         }
                         if (!NMC_IN_BOUNDS(g.dbg, P, N2, kDbgHistory)) break;
                         if (P < 64) done0 |= 1ull << P; else done1 |= 1ull << (P - 64);
-                        if (tid == 0) nd->prow[c] = P;
+                        if (tid == lead) nd->prow[c] = P;
                         // The warp's rows r = warp + nwarps i, 32 at a time: lane i forms row i's multiplier
                         // (one FP64 instruction for 32 rows instead of one per row), the rows are updated one
                         // after another with all lanes along j, and then lane i reads row i's new entry of
@@ -401,11 +425,8 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                             }
                             __syncwarp();
                             if (ract && c + 1 < N2) {
-                                const double v = fabs(Mt[rl * LDM + c + 1]);
-                                if (v == v) {
-                                    const long long key = __double_as_longlong(v);
-                                    if (key > bkey) { bkey = key; brow = rl; }
-                                }
+                                const long long key = (long long)abs_bits(Mt[rl * LDM + c + 1]);
+                                if (key > bkey && key <= (long long)kInfBits) { bkey = key; brow = rl; }
                             }
                         }
                         long long wkey = bkey;
@@ -415,11 +436,10 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                         }
                         const int wrow = (int)__reduce_min_sync(kFull, (unsigned)(bkey == wkey && wkey >= 0 ? brow : 0x7fffffff));
                         if (lane == 0) {
-                            const double nb = wkey >= 0 ? __longlong_as_double(wkey) : -1.0;
                             const int ni = wkey >= 0 ? wrow : 0;
-                            nd->cv[bsel ^ 1][warp] = nb;
+                            nd->cv[bsel ^ 1][warp] = wkey;
                             nd->ci[bsel ^ 1][warp] = ni;
-                            nd->cip[bsel ^ 1][warp] = nb > 0.0 ? 1.0 / Mt[ni * LDM + c + 1] : 0.0;
+                            nd->cip[bsel ^ 1][warp] = wkey > 0 ? 1.0 / Mt[ni * LDM + c + 1] : 0.0;
                         }
                         __syncthreads();
                     }
@@ -484,7 +504,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                     if (a.gH_in)
                         for (int c = 0; c < 3; ++c) a.gH_in[o * 3 + c] = gH[c] * fI;
                 }
-                if (tid == 0) {
+                if (tid == lead) {
                     a.gYe_in[n] = be * nd->deps_dYe_star + by;
                     a.gT_in[n] = be * nd->deps_dT_star;
                     if (a.gscale)
@@ -501,14 +521,14 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                 if (a.gH_in)
                     for (int c = 0; c < 3; ++c) a.gH_in[o * 3 + c] = 0.0;
             }
-            if (tid == 0) {
+            if (tid == lead) {
                 a.gYe_in[n] = 0.0;
                 a.gT_in[n] = 0.0;
                 if (a.gscale)
                     for (int k = 0; k < 4; ++k) a.gscale[n * 4 + k] = 0.0;
             }
         }
-        if (tid == 0 && a.status) a.status[n] = (uint32_t)nd->status;
+        if (tid == lead && a.status) a.status[n] = (uint32_t)nd->status;
         __syncthreads();
     }
 }

@@ -184,9 +184,9 @@ __device__ inline double eos_temperature_warp(double rho, double nb, double f, d
     return T;
 }
 
-__device__ __forceinline__ double eos_deps_dye(double rho, double T, double Ye) {
+// d eps / dYe at fixed rho, T
+__device__ __forceinline__ double eos_deps_dye_at_mu(double T, double mu) {
     const double pi2 = kPi * kPi;
-    const double mu = eos_mu_e(rho, T, Ye);
     const double mu2 = mu * mu, T2 = T * T;
     return kMeVErg / kMB * 3.0 * mu * (mu2 + pi2 * T2) / (3.0 * mu2 + pi2 * T2);
 }
