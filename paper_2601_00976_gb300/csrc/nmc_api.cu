@@ -374,6 +374,12 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         if (e != cudaSuccess) rc = NMC_ENOMEM;
         else { ctx->allocations.push_back(p); ctx->queue = static_cast<int*>(p); }
     }
+    if (rc == NMC_OK) {
+        void* p = nullptr;
+        e = cudaMalloc(&p, kOrderMax * sizeof(int));
+        if (e != cudaSuccess) rc = NMC_ENOMEM;
+        else { ctx->allocations.push_back(p); ctx->order = static_cast<int*>(p); }
+    }
 #ifdef NMC_DEBUG
     if (rc == NMC_OK) {   // the bounds-check error word, cleared
         void* p = nullptr;
@@ -400,6 +406,7 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         if (e == cudaSuccess) e = preload_fused_f64_m5();
         if (e == cudaSuccess) e = preload_fused_f32_m3();
         if (e == cudaSuccess) e = preload_fused_f32_m5();
+        if (e == cudaSuccess) e = preload_order();
         if (e != cudaSuccess) rc = NMC_ECUDA;
     }
     if (rc == NMC_OK) {
@@ -475,6 +482,7 @@ int collision_solve(nmc_ctx* ctx, const nmc_params* params, int64_t n, const dou
     a.J_out = J_out; a.H_out = H_out; a.Ye_out = Ye_out; a.eps_out = eps_out; a.T_out = T_out;
     a.n_outer = n_outer; a.n_inner = n_inner; a.status = status;
     a.queue = ctx->queue;
+    a.order = ctx->order;
     if (params->mode == NMC_MODE_PLAIN) return launch_plain(ctx, a, static_cast<cudaStream_t>(stream));
     return launch_fused(ctx, a, static_cast<cudaStream_t>(stream));
 }
@@ -505,6 +513,7 @@ int collision_solve_v(nmc_ctx* ctx, const nmc_params* params, int64_t n, const d
     a.J_out = J_out; a.H_out = H_out; a.Ye_out = Ye_out; a.eps_out = eps_out; a.T_out = T_out;
     a.n_outer = n_outer; a.n_inner = n_inner; a.status = status;
     a.queue = ctx->queue;
+    a.order = ctx->order;
     return launch_velocity(ctx, a, v_in, v_out, freeze_velocity ? 1 : 0, v_floor, static_cast<cudaStream_t>(stream));
 }
 
@@ -545,6 +554,7 @@ int nmc_autotune(nmc_ctx* ctx, const nmc_params* params, int64_t n, const double
     a.J_out = J_out; a.H_out = H_out; a.Ye_out = Ye_out; a.eps_out = eps_out; a.T_out = T_out;
     a.n_outer = n_outer; a.n_inner = n_inner; a.status = status;
     a.queue = ctx->queue;
+    a.order = ctx->order;
     return autotune_fused(ctx, a, static_cast<cudaStream_t>(stream), chosen, ms);
 }
 

@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
     for (;;) {
         if (tid == 0) {
             long long nn = atomicAdd(a.queue, 1);
+            if (a.order && nn < a.n) nn = a.order[nn];
 #ifdef NMC_DEBUG
             if (g.dbg && *reinterpret_cast<volatile unsigned*>(g.dbg) != 0u) nn = a.n;   // a check failed: stop
 #endif
@@ -738,9 +739,9 @@ static int launch_impl(nmc_ctx* ctx, SolveArgs a, cudaStream_t stream, int grid_
         return set_error(ctx, NMC_EUNSUPPORTED, "fused kernel cannot be resident with this shape");
     long long grid = (long long)per_sm * ctx->num_sms * grid_pct / 100;
     if (grid < ctx->num_sms) grid = ctx->num_sms;
+    const int rc = start_queue(ctx, a, grid, stream);
+    if (rc != NMC_OK) return rc;
     if (grid > a.n) grid = a.n;
-    e = cudaMemsetAsync(a.queue, 0, sizeof(int), stream);
-    if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
     kern<<<(unsigned)grid, threads, smem, stream>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("fused kernel launch: ") + cudaGetErrorString(e));

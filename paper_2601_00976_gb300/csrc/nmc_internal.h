@@ -172,6 +172,7 @@ struct SolveArgs {
     int32_t* n_inner;
     uint32_t* status;
     int* queue;
+    int* order;   // the context's node order (kOrderMax entries), null: nodes in index order
     // shared-memory carve (byte offsets)
     int off_phi, off_ann, off_vec, off_red, off_node;
 };
@@ -239,6 +240,7 @@ struct nmc_ctx {
     // device allocations owned by the context
     std::vector<void*> allocations;
     int* queue = nullptr;
+    int* order = nullptr;   // node order of the persistent kernels (kOrderMax entries)
     // plain mode: chunk size (nodes) and its scratch, grown on demand and kept
     long long plain_chunk = 1LL << 17;
     void* plain_scratch = nullptr;
@@ -268,6 +270,10 @@ int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long 
 size_t fused_smem_bytes(const nmc_ctx* ctx, int maxm, bool mixed, SolveArgs* a);
 int launch_adjoint(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream);
 int launch_plain(nmc_ctx* ctx, const SolveArgs& a, cudaStream_t stream);
+// Clears the work queue of a launch with `resident` blocks and, where it pays, orders the nodes (a.order stays set)
+constexpr int kOrderMax = 1 << 16;
+int start_queue(nmc_ctx* ctx, SolveArgs& a, long long resident, cudaStream_t stream);
+cudaError_t preload_order();
 int launch_velocity(nmc_ctx* ctx, const SolveArgs& a, const double* v_in, double* v_out, int freeze,
                     double v_floor, cudaStream_t stream);
 int launch_c2p(nmc_ctx* ctx, long long n, const double* N, const double* G, const double* v, double tol,

@@ -215,7 +215,10 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
         for (int c = 0; c < 4; ++c) { Fh[j][c] = 0.0; Qh[j][c] = 0.0; }
 
     for (;;) {
-        if (tid == 0) nd->node = atomicAdd(a.queue, 1);
+        if (tid == 0) {
+            const int nn = atomicAdd(a.queue, 1);
+            nd->node = a.order && nn < a.n ? a.order[nn] : nn;
+        }
         __syncthreads();
         const long long n = nd->node;
         if (n >= a.n) break;
@@ -628,9 +631,9 @@ int launch_velocity_impl(nmc_ctx* ctx, VelArgs va, size_t smem, int threads, cud
     if (e != cudaSuccess || per_sm < 1)
         return set_error(ctx, NMC_EUNSUPPORTED, "velocity kernel cannot be resident with this shape");
     long long grid = (long long)per_sm * ctx->num_sms;
+    const int rc = start_queue(ctx, va.a, grid, stream);
+    if (rc != NMC_OK) return rc;
     if (grid > va.a.n) grid = va.a.n;
-    e = cudaMemsetAsync(va.a.queue, 0, sizeof(int), stream);
-    if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
     kern<<<(unsigned)grid, threads, smem, stream>>>(va);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("velocity kernel launch: ") + cudaGetErrorString(e));
