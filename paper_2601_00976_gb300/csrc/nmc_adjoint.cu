@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
             Tk = lane_value(Tk, 0);
             const double mu = eos_mu_e_warp(y1 * rho / kMB, Tk);
             double e, de;
-            eos_eps_at_mu_warp(nd->nb, nd->f, Tk, mu, &e, &de);
+            eos_eps_at_mu_warp<true>(nd->nb, nd->f, Tk, mu, &e, &de);
             if (ln == 0) {
                 nd->y[0] = y0;
                 nd->y[1] = y1;
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                 const double gT = a.gT ? a.gT[n] : 0.0;
                 const double ge = a.geps ? a.geps[n] : 0.0, gy = a.gYe ? a.gYe[n] : 0.0;
                 nd->g_y[0] = ge + gT / de;
-                nd->g_y[1] = gy - gT * eos_deps_dye_at_mu(Tk, mu) / de;
+                nd->g_y[1] = gy - gT * eos_deps_dye_at_mu<true>(Tk, mu) / de;
                 nd->h[0] = h0;
                 nd->h[1] = h1;
                 if (!(isfinite(nd->g_y[0]) && isfinite(nd->g_y[1]))) { nd->status |= NMC_NONFINITE; nd->bad = 1; }

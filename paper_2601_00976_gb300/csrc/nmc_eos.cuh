@@ -85,7 +85,9 @@ __device__ __forceinline__ double eos_mu_e_warp(double ne, double T, double* rT 
 }
 
 // eos_eps_at_mu with nb = rho / m_B and f = (MeV in erg) / rho.  The products and sums are written as the
-// fused operations the compiler contracts them to in eos_eps_at_mu, so that both round alike.
+// fused operations the compiler contracts them to in eos_eps_at_mu, so that both round alike; kShared: where
+// pi^2 T^2 is shared with eos_deps_dye_at_mu, it is rounded before it is added.
+template <bool kShared = false>
 __device__ __forceinline__ void eos_eps_at_mu_warp(double nb, double f, double T, double mu, double* eps, double* deps) {
     const int ln = threadIdx.x & 31;
     const double pi2 = kPi * kPi;
@@ -94,7 +96,7 @@ __device__ __forceinline__ void eos_eps_at_mu_warp(double nb, double f, double T
     double num = 7.0 * pi2 * T2 * T2, den = 60.0;
     if (ln == 1) { num = mu2 * mu2; den = 4.0 * pi2; }
     if (ln == 2) { num = pi2 / 15.0 * T2 * T2; den = hc3; }
-    if (ln == 3) { num = -2.0 * pi2 * T * mu; den = __fma_rn(pi2, T2, __dmul_rn(3.0, mu2)); }
+    if (ln == 3) { num = -2.0 * pi2 * T * mu; den = kShared ? __fma_rn(3.0, mu2, __dmul_rn(pi2, T2)) : __fma_rn(pi2, T2, __dmul_rn(3.0, mu2)); }
     if (ln == 4) { num = 7.0 * pi2 * T2 * T; den = 15.0; }
     if (ln == 5) { num = mu2 * mu; den = pi2; }
     if (ln == 6) { num = 4.0 * pi2 / 15.0 * T2 * T; den = hc3; }
@@ -184,11 +186,15 @@ __device__ inline double eos_temperature_warp(double rho, double nb, double f, d
     return T;
 }
 
-// d eps / dYe at fixed rho, T
+// d eps / dYe at fixed rho, T (kShared: see eos_eps_at_mu_warp)
+template <bool kShared = false>
 __device__ __forceinline__ double eos_deps_dye_at_mu(double T, double mu) {
     const double pi2 = kPi * kPi;
     const double mu2 = mu * mu, T2 = T * T;
-    return kMeVErg / kMB * 3.0 * mu * (mu2 + pi2 * T2) / (3.0 * mu2 + pi2 * T2);
+    const double t = __dmul_rn(pi2, T2);
+    const double num = kShared ? __dadd_rn(mu2, t) : __fma_rn(pi2, T2, mu2);
+    const double den = kShared ? __fma_rn(3.0, mu2, t) : __fma_rn(pi2, T2, __dmul_rn(3.0, mu2));
+    return kMeVErg / kMB * 3.0 * mu * num / den;
 }
 
 // ---- FP32 variants for the mixed-precision path ----
