@@ -56,7 +56,7 @@ struct VelNode {
     double qh[kMaxOuterMem][kNy], fh[kMaxOuterMem][kNy];
     double G[3][3];
     double alpha[3];
-    double t2[kMaxSpecies];               // Algorithm 2's thresholds on the squared changes
+    VoteLimit lim[kMaxSpecies];           // Algorithm 2's thresholds
     double sp_out[kMaxSpecies * 4];
     double blk_out[16];
     OpacState op;
@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
     const double W2q = act ? g.w2[q] : 0.0;
     const double W3q = act ? g.w3[q] : 0.0;
     const double Wt = act ? g.wt[q] : 0.0;
+    const float Wt_f = act ? g.wt_f[q] : 0.0f;
     double Fh[3][4], Qh[3][4];
     for (int j = 0; j < 3; ++j)
         for (int c = 0; c < 4; ++c) { Fh[j][c] = 0.0; Qh[j][c] = 0.0; }
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                 const int sp = tid - lead;   // one species per lane of the lead warp
                 if (sp >= 0 && sp < NS) {
                     const double fl = P.norm_floor * sqrt(g.sum_wt);
-                    nd->t2[sp] = square_threshold(P.tol_inner * fmax(sqrt(nd->sp_out[sp]), fl));
+                    nd->lim[sp] = vote_limit(P.tol_inner * fmax(sqrt(nd->sp_out[sp]), fl));
                 }
             }
             auto publish = [&](const double (&Mv)[4]) {
@@ -473,11 +474,11 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                 publish(Mn);
                 int vote = 1;
                 {   // Algorithm 2
-                    double v[4];
-                    for (int c = 0; c < 4; ++c) { const double d = Mn[c] - M[c]; v[c] = Wt * d * d; }
+                    double d[4];
+                    for (int c = 0; c < 4; ++c) d[c] = Mn[c] - M[c];
                     if (act && !(is_finite(Mn[0]) && is_finite(Mn[1]) && is_finite(Mn[2]) && is_finite(Mn[3])))
                         nd->bad = 1;
-                    vote = species_vote(v, nd->t2, nd->t2, NEP, NS, s, red);
+                    vote = species_vote_fp64(d, Wt, Wt_f, nd->lim, NEP, NS, s, red);
                 }
                 const bool conv = __syncthreads_and(vote) != 0;
                 const bool bad = *reinterpret_cast<volatile int*>(&nd->bad) != 0;
