@@ -282,7 +282,7 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         double swt = 0.0;
         for (int gq = 0; gq < Q; ++gq) {
             const double eg = c + h * xg[gq];
-            pe[el * Q + gq] = eg;
+            pe[gq * n_elem + el] = eg;   // the element fastest: a warp's lanes take neighbouring elements
             wt[gq] = wg[gq] * eg * eg * h;          // eps^2 d eps
             swt += wt[gq];
             for (int p = 0; p < nq; ++p) L[p * Q + gq] = lagrange(xi, p, xg[gq]);
@@ -296,9 +296,9 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
             for (int gq = 0; gq < Q; ++gq) {
                 double v = 0.0;
                 for (int r = 0; r < nq; ++r) v += M[p * nq + r] * wt[gq] * L[r * Q + gq];
-                pc[(el * nq + p) * Q + gq] = v;
+                pc[(p * Q + gq) * n_elem + el] = v;
             }
-        for (int gq = 0; gq < Q; ++gq) pa[el * Q + gq] = wt[gq] / swt;
+        for (int gq = 0; gq < Q; ++gq) pa[gq * n_elem + el] = wt[gq] / swt;
     }
     DevGrid& g = ctx->g;
     g.ns = ns;

@@ -824,39 +824,41 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
         // NES kernel reads across the species.
         // The ns n_elem tasks are dealt out to consecutive threads from the lead warp on: one full warp
         // instead of several partly empty ones (an instruction costs the same), on SMSPs that change
-        // with the node.
+        // with the node.  Operators and Fermi--Dirac values are laid out with the element fastest, so that
+        // the lanes' loads are coalesced and free of bank conflicts.
         constexpr int kHalfQ = kProjQuad / 2;
         const int task0 = tid >= lead ? tid - lead : tid - lead + (int)blockDim.x;
         for (int task = task0; task < NS * g.n_elem; task += blockDim.x) {
             const int s = task / g.n_elem, e = task - s * g.n_elem;
             const int nq = g.nq;
-            if (!NMC_IN_BOUNDS(g.dbg, ((long long)e * nq + nq - 1) * kProjQuad + kProjQuad - 1,
+            if (!NMC_IN_BOUNDS(g.dbg, ((long long)nq * kProjQuad - 1) * g.n_elem + e,
                                (long long)g.n_elem * nq * kProjQuad, kDbgProj) ||
                 !NMC_IN_BOUNDS(g.dbg, (long long)s * NEP + e * nq + nq - 1, (long long)NS * NEP, kDbgSmemVec))
                 continue;
             const int sfd = s < 2 ? s : 2;   // the heavy flavours' Fermi--Dirac values are species 2's
-            const R* f = fq + sfd * nqp + e * kProjQuad;
-            const R* fc = fq + (NS + sfd) * nqp + e * kProjQuad;
+            const int ns_e = g.n_elem;   // step between an element's quadrature points
+            const R* f = fq + sfd * nqp + e;
+            const R* fc = fq + (NS + sfd) * nqp + e;
             R avg = 0, avgc = 0, coef[kMaxNq] = {0, 0, 0}, coefc[kMaxNq] = {0, 0, 0};
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 R pa[kHalfQ], pc[kMaxNq][kHalfQ];
 #pragma unroll
                 for (int gq = 0; gq < kHalfQ; ++gq) {
-                    const int qa = e * kProjQuad + h * kHalfQ + gq;
+                    const int qa = (h * kHalfQ + gq) * ns_e + e;
                     pa[gq] = kMixed ? (R)__ldg(g.proj_a_f + qa) : (R)__ldg(g.proj_a + qa);
 #pragma unroll
                     for (int pp = 0; pp < kMaxNq; ++pp) {
-                        const int o = (e * nq + min(pp, nq - 1)) * kProjQuad + h * kHalfQ + gq;
+                        const int o = (min(pp, nq - 1) * kProjQuad + h * kHalfQ + gq) * ns_e + e;
                         pc[pp][gq] = kMixed ? (R)__ldg(g.proj_c_f + o) : (R)__ldg(g.proj_c + o);
                     }
                 }
 #pragma unroll
                 for (int gq = 0; gq < kHalfQ; ++gq) {
-                    const R fv = f[h * kHalfQ + gq];
+                    const R fv = f[(h * kHalfQ + gq) * ns_e];
                     avg += pa[gq] * fv;
                     R fcv = 0;
-                    if (kMixed) { fcv = fc[h * kHalfQ + gq]; avgc += pa[gq] * fcv; }
+                    if (kMixed) { fcv = fc[(h * kHalfQ + gq) * ns_e]; avgc += pa[gq] * fcv; }
 #pragma unroll
                     for (int pp = 0; pp < kMaxNq; ++pp) {
                         if (pp >= nq) break;

@@ -97,9 +97,9 @@ struct DevGrid {
     const double* w2;      // [ne]
     const double* w3;      // [ne]
     const double* lneps;   // [ne] ln eps (opacity_interp energy axis)
-    const double* proj_e;  // [n_elem][Q] quadrature energies
-    const double* proj_c;  // [n_elem][nq][Q] projection operator (mass^-1 * basis * weights)
-    const double* proj_a;  // [n_elem][Q] eps^2-weighted cell-average weights
+    const double* proj_e;  // [Q][n_elem] quadrature energies
+    const double* proj_c;  // [nq][Q][n_elem] projection operator (mass^-1 * basis * weights)
+    const double* proj_a;  // [Q][n_elem] eps^2-weighted cell-average weights
     const double* wt;      // [ne] W2 / (4 pi / (hc)^3) = w eps^2 Delta eps  [MeV^3]
     // FP32 copies for the mixed-precision kernel
     const float* proj_e_f;   // proj_e as double-floats: high words
