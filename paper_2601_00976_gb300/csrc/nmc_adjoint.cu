@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
             double e = 0.0, de = 0.0, mu = 0.0;
             if (okin) {
                 mu = eos_mu_e_warp(lane_value(d, 1), T);
-                eos_eps_at_mu_warp(nb, f, T, mu, &e, &de);
+                eos_eps_at_mu_warp<false, false>(nb, f, T, mu, &e, &de);
             }
             const double dy = okin ? eos_deps_dye_at_mu(T, mu) : 0.0;
             if (lane < 4) {
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
             Tk = lane_value(Tk, 0);
             const double mu = eos_mu_e_warp(y1 * rho / kMB, Tk);
             double e, de;
-            eos_eps_at_mu_warp<true>(nd->nb, nd->f, Tk, mu, &e, &de);
+            eos_eps_at_mu_warp<true, false>(nd->nb, nd->f, Tk, mu, &e, &de);
             if (ln == 0) {
                 nd->y[0] = y0;
                 nd->y[1] = y1;

@@ -138,6 +138,28 @@ __device__ __forceinline__ void warp_partials(T (&v)[K], void* scratch) {
     if ((lane & ((32 >> kFoldLevels<K>) - 1)) == 0 && k < K) red[w * K + k] = v[0];
 }
 
+// The warps' partials of value k added in warp order.  Blocks of 4 and 8 warps, the usual ones, take
+// their own code: this sum is on every inner iteration's critical path, and the loop's bookkeeping
+// between dependent loads and additions cost the mixed solve 1-2%.
+template <int K, int NW, typename T>
+__device__ __forceinline__ T add_partials_of(const T* red, int k) {
+    T p[NW], s = 0;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) p[i] = red[i * K + k];
+#pragma unroll
+    for (int i = 0; i < NW; ++i) s += p[i];
+    return s;
+}
+
+template <int K, typename T>
+__device__ __forceinline__ T add_partials(const T* red, int k, int nw) {
+    if (nw == 8) return add_partials_of<K, 8>(red, k);
+    if (nw == 4) return add_partials_of<K, 4>(red, k);
+    T s = 0;
+    for (int i = 0; i < nw; ++i) s += red[i * K + k];
+    return s;
+}
+
 // Sum K values over the whole block; result in out[0..K).
 template <int K, typename T>
 __device__ __forceinline__ void block_sum(T (&v)[K], void* scratch, T* out) {
@@ -519,6 +541,46 @@ __device__ __forceinline__ void anderson3_warp(double e, int n, double& c0, doub
     }
 }
 
+// The same from FP32 entries (lane k < 5: entry k), exactly those of anderson3_warp on the entries widened:
+// the exchange, the selections and the tests run on single words, and only the four operands a lane
+// multiplies are widened.  The other warps wait for this chain in every inner iteration.
+__device__ __forceinline__ void anderson3_warp(float e, int n, double& c0, double& c1, double& cL) {
+    const int lane = threadIdx.x & 31;
+    c0 = 0.0;
+    c1 = 0.0;
+    cL = 1.0;
+    if (n == 2) {
+        const float a00 = __shfl_sync(kFull, e, 0), a01 = __shfl_sync(kFull, e, 1);
+        const float a11 = __shfl_sync(kFull, e, 2), r0 = __shfl_sync(kFull, e, 3);
+        const float r1 = __shfl_sync(kFull, e, 4);
+        const float dmax = fmaxf(fabsf(a00), fabsf(a11));
+        if (!(dmax > 0.0f) || !isfinite(dmax)) return;
+        const bool sw = fabsf(a01) > fabsf(a00);   // column 0 with partial pivoting (A is symmetric)
+        const float p0 = sw ? a01 : a00, p1 = sw ? a11 : a01, pr = sw ? r1 : r0;
+        const float q0 = sw ? a00 : a01, q1 = sw ? a01 : a11, qr = sw ? r0 : r1;
+        const int ed = (__float_as_int(dmax) >> 23) & 0xff, ep = (__float_as_int(p0) >> 23) & 0xff;
+        const bool plain = ed > 0 && ep > 0 && ep < 255;   // normal: the exponents decide where they can
+        if (!(plain && ep >= ed - 45) && !(fabs((double)p0) > 1e-14 * (double)dmax)) return;
+        const double x = widen(lane == 2 ? pr : p0), y = widen(lane == 1 ? qr : q1);
+        const double z = widen(lane == 2 ? p1 : q0), w = widen(lane == 0 ? p1 : (lane == 1 ? pr : qr));
+        const double t = x * y - z * w;
+        const double det = __shfl_sync(kFull, t, 0);
+        const int et = exponent_of(det);
+        if (!(plain && normal_exponent(et) && et >= ed + ep + 725) &&
+            !abs_gt(det, 1e-14 * (double)dmax * fabs((double)p0))) return;
+        const double gm = t * (1.0 / det);
+        const double gm1 = __shfl_sync(kFull, gm, 1), gm0 = __shfl_sync(kFull, gm, 2);
+        const double sum = gm0 + gm1;
+        if (is_finite(sum)) { c0 = gm0; c1 = gm1; cL = 1.0 - sum; }
+    } else if (n == 1) {
+        const double a00 = widen(__shfl_sync(kFull, e, 0)), r0 = widen(__shfl_sync(kFull, e, 3));
+        if (abs_bits(a00) - 1 < kInfBits - 1) {
+            const double gam = r0 / a00;
+            if (is_finite(gam)) { c0 = gam; cL = 1.0 - gam; }
+        }
+    }
+}
+
 // Coefficient of history column j (0..2, newest last) from anderson3_warp's
 // (c0, c1, cL): n = 2 -> (g0, g1, L) = (0, 1, 2); n = 1 -> (g0, L) = (1, 2).
 __device__ __forceinline__ double anderson3_coef(int j, int n, double c0, double c1, double cL) {
@@ -729,16 +791,16 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
             if (ln < 8) { if constexpr (kMixed) os->w8_f[ln] = w3; else os->w8[ln] = w3; }
             if (ln < 4) { if constexpr (kMixed) os->w4_f[ln] = w2; else os->w4[ln] = w2; }
         }
+        if (ln < 4) {   // FP32 tables carry 4 pi / (hc)^3
+            const double pre = (kMixed || ln < 2 ? dtau : dtau * kCW) * sc[ln];
+            if constexpr (kMixed) os->pre_f[ln] = narrow(pre);
+            else os->pre[ln] = pre;
+        }
         if (ln == 0) {
             os->tinv = tinv;
             os->eta_e = eta_e;
             for (int sp = 0; sp < kMaxSpecies; ++sp) os->mu[sp] = sp == 0 ? mnu : (sp == 1 ? -mnu : 0.0);
             if (any_cl) *status |= NMC_TABLE_CLAMP;
-            const double unit = kMixed ? dtau : dtau * kCW;   // FP32 tables carry 4 pi/(hc)^3
-            os->pre[0] = dtau * sc[0];
-            os->pre[1] = dtau * sc[1];
-            os->pre[2] = unit * sc[2];
-            os->pre[3] = unit * sc[3];
             if (kMixed) {
                 const F2 m2 = f2_from(mnu), t2 = f2_from(tinv);
                 for (int sp = 0; sp < kMaxSpecies; ++sp) {
@@ -747,7 +809,6 @@ __device__ void compute_opacities(const DevGrid& g, const DevTables& tb, const n
                 }
                 os->tinv_h = t2.h;
                 os->tinv_l = t2.l;
-                for (int k = 0; k < 4; ++k) os->pre_f[k] = (float)os->pre[k];
             }
         }
     }

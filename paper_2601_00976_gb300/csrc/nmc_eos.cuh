@@ -87,19 +87,31 @@ __device__ __forceinline__ double eos_mu_e_warp(double ne, double T, double* rT 
 // eos_eps_at_mu with nb = rho / m_B and f = (MeV in erg) / rho.  The products and sums are written as the
 // fused operations the compiler contracts them to in eos_eps_at_mu, so that both round alike; kShared: where
 // pi^2 T^2 is shared with eos_deps_dye_at_mu, it is rounded before it is added.
-template <bool kShared = false>
+// kLanes: numerators formed lane-parallel as well (not in the adjoint, whose register budget it overruns).
+template <bool kShared = false, bool kLanes = true>
 __device__ __forceinline__ void eos_eps_at_mu_warp(double nb, double f, double T, double mu, double* eps, double* deps) {
     const int ln = threadIdx.x & 31;
     const double pi2 = kPi * kPi;
     const double hc3 = kHbarC * kHbarC * kHbarC;
     const double T2 = T * T, mu2 = mu * mu;
-    double num = 7.0 * pi2 * T2 * T2, den = 60.0;
-    if (ln == 1) { num = mu2 * mu2; den = 4.0 * pi2; }
-    if (ln == 2) { num = pi2 / 15.0 * T2 * T2; den = hc3; }
-    if (ln == 3) { num = -2.0 * pi2 * T * mu; den = kShared ? __fma_rn(3.0, mu2, __dmul_rn(pi2, T2)) : __fma_rn(pi2, T2, __dmul_rn(3.0, mu2)); }
-    if (ln == 4) { num = 7.0 * pi2 * T2 * T; den = 15.0; }
-    if (ln == 5) { num = mu2 * mu; den = pi2; }
-    if (ln == 6) { num = 4.0 * pi2 / 15.0 * T2 * T; den = hc3; }
+    // numerators (k x) y, denominators
+    double k = 7.0 * pi2, x = T2, y = T2, den = 60.0;
+    if (ln == 1) { k = 1.0; x = mu2; y = mu2; den = 4.0 * pi2; }
+    if (ln == 2) { k = pi2 / 15.0; den = hc3; }
+    if (ln == 3) { k = -2.0 * pi2; x = T; y = mu; den = kShared ? __fma_rn(3.0, mu2, __dmul_rn(pi2, T2)) : __fma_rn(pi2, T2, __dmul_rn(3.0, mu2)); }
+    if (ln == 4) { y = T; den = 15.0; }
+    if (ln == 5) { k = 1.0; x = mu2; y = mu; den = pi2; }
+    if (ln == 6) { k = 4.0 * pi2 / 15.0; y = T; den = hc3; }
+    double num = __dmul_rn(__dmul_rn(k, x), y);
+    if (!kLanes) {
+        num = 7.0 * pi2 * T2 * T2;
+        if (ln == 1) num = mu2 * mu2;
+        if (ln == 2) num = pi2 / 15.0 * T2 * T2;
+        if (ln == 3) num = -2.0 * pi2 * T * mu;
+        if (ln == 4) num = 7.0 * pi2 * T2 * T;
+        if (ln == 5) num = mu2 * mu;
+        if (ln == 6) num = 4.0 * pi2 / 15.0 * T2 * T;
+    }
     const double d = num / den;
     const double u1 = lane_value(d, 0), u2 = lane_value(d, 1), ug = lane_value(d, 2), dmu = lane_value(d, 3);
     const double v1 = lane_value(d, 4), v2 = lane_value(d, 5), dug = lane_value(d, 6);

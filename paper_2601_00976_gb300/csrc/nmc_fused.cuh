@@ -268,6 +268,8 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                 compute_opacities<R>(g, a.tb, P, nd->rho, nd->T, nd->y[1], nd->dtau, nd->sc, ob, &nd->op,
                                      &nd->status, chiab, sig, deq, deqc, lead, nd->mu_T);
             NMC_TRACE_TICK(kTrOpac);
+            // mixed: from here on deqc carries W~ / (1 - D^Eq), its only use
+            if (kMixed && (k == 1 || !P.semi_implicit)) deqc = Wt / deqc;
             if constexpr (kMixed) {
                 const double c1 = (double)Wt, c2 = c1 * (double)chiab;
                 A0x = f2_from(c1 * Dsd + c2 * (double)deq);
@@ -305,7 +307,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                     if constexpr (kMixed) {
                         myW1D = Wt * hole;
                         myAW1D = aq * Wt * hole;
-                        myWdev = __fadd_rn(__fsub_rn(D2.h, (float)deq), D2.l) * (Wt / deqc);
+                        myWdev = __fadd_rn(__fsub_rn(D2.h, (float)deq), D2.l) * deqc;
                         xw[sq] = make_float2(Wt * D32, myWdev);
                         yz[sq].x = myW1D;
                         yz[(s ^ 1) * NEP + q].y = myAW1D;
@@ -532,13 +534,10 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                         const int k = tid & 31;
                         const R* pr = reinterpret_cast<const R*>(red);
                         R sk = 0;
-                        if (k < K)
-                            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) sk += pr[i * K + k];
-                        double e;
-                        if constexpr (kMixed) e = widen(sk);
-                        else e = gram3_update_warp<3>(nd->G, sk, m);
+                        if (k < K) sk = add_partials<K, R>(pr, k, blockDim.x >> 5);
                         double c0, c1, cL;
-                        anderson3_warp(e, m - 1, c0, c1, cL);
+                        if constexpr (kMixed) anderson3_warp(sk, m - 1, c0, c1, cL);
+                        else anderson3_warp(gram3_update_warp<3>(nd->G, sk, m), m - 1, c0, c1, cL);
                         if (k < 3) {
                             const double a = anderson3_coef(k, m - 1, c0, c1, cL);
                             if constexpr (kMixed) nd->alpha_f[k] = narrow(a);

@@ -455,8 +455,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
                         const int kk = tid & 31;
                         const double* pr = reinterpret_cast<const double*>(red);
                         double sk = 0.0;
-                        if (kk < 3)
-                            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) sk += pr[i * 3 + kk];
+                        if (kk < 3) sk = add_partials<3, double>(pr, kk, blockDim.x >> 5);
                         const double e = gram3_update_warp<3>(nd->G, sk, m);
                         double c0, c1, cL;
                         anderson3_warp(e, m - 1, c0, c1, cL);
