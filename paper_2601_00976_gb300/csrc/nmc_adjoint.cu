@@ -367,10 +367,10 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                     // tracks, among the rows it has just updated, the largest |entry| of the next column
                     // (lane 0 updates that column), so one barrier per column publishes both the updated
                     // rows and the next pivot's candidates.  Every thread then picks the same pivot.
-                    unsigned long long done0 = 0ull, done1 = 0ull;   // eliminated pivot rows (2 ne <= 128)
-                    auto is_done = [&](int r) {
-                        return ((r < 64 ? done0 >> r : done1 >> (r - 64)) & 1ull) != 0ull;
-                    };
+                    // This warp's rows warp + nwarps i (at most 32 of them: 2 ne rows, ns nep >= 2 ne threads), those
+                    // not yet a pivot row as a bit mask over i.
+                    const int rows_w = (N2 - warp + nwarps - 1) / nwarps;
+                    unsigned alive = rows_w >= 32 ? kFull : (1u << rows_w) - 1u;
                     if (lane == 0) {   // column 0's candidates
                         double nip = 0.0;
                         long long nb = -1;
@@ -400,34 +400,43 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                             break;
                         }
                         if (!NMC_IN_BOUNDS(g.dbg, P, N2, kDbgHistory)) break;
-                        if (P < 64) done0 |= 1ull << P; else done1 |= 1ull << (P - 64);
+                        if (P % nwarps == warp) alive &= ~(1u << (P / nwarps));
                         if (tid == lead) nd->prow[c] = P;
-                        // The warp's rows r = warp + nwarps i, 32 at a time: lane i forms row i's multiplier
-                        // (one FP64 instruction for 32 rows instead of one per row), the rows are updated one
-                        // after another with all lanes along j, and then lane i reads row i's new entry of
+                        // Lane i forms the multiplier of the warp's row i (one FP64 instruction for all its rows), the
+                        // active rows are updated two at a time with all lanes along j (so that one row's loads and
+                        // FP64 operations overlap the other's), and then lane i reads row i's new entry of
                         // column c + 1.  The warp's candidate is the largest |entry|, the smallest row among
                         // equals (as a scan in row order would pick): |entry| compared as the integer of its
                         // bits (order-preserving for non-negative doubles; NaN is no candidate), so the
                         // search issues no FP64 compare.
-                        const int rows_w = (N2 - warp + nwarps - 1) / nwarps;
-                        long long bkey = -1;   // best |entry| bits of this lane's rows (-1: none)
-                        int brow = 0;
-                        for (int i0 = 0; i0 < rows_w; i0 += 32) {
-                            const int rl = warp + nwarps * (i0 + lane);
-                            const bool ract = i0 + lane < rows_w && !is_done(rl);
-                            const double lmul = ract ? Mt[rl * LDM + c] * ip : 0.0;
-                            const int ng = rows_w - i0 < 32 ? rows_w - i0 : 32;
-                            for (int k = 0; k < ng; ++k) {
-                                const double l = __shfl_sync(kFull, lmul, k);
-                                const int r = warp + nwarps * (i0 + k);
-                                if (is_done(r)) continue;
-                                for (int j = c + 1 + lane; j < N2 + 3; j += 32) Mt[r * LDM + j] -= l * Mt[P * LDM + j];
+                        const int rl = warp + nwarps * lane;
+                        const bool ract = (alive >> lane) & 1u;
+                        const double lmul = ract ? Mt[rl * LDM + c] * ip : 0.0;
+                        const double* prow = Mt + P * LDM;
+                        for (unsigned m = alive; m != 0u;) {
+                            const int k0 = __ffs(m) - 1;
+                            m &= m - 1;
+                            const int k1 = m != 0u ? __ffs(m) - 1 : k0;
+                            m &= m - 1;
+                            double* row0 = Mt + (warp + nwarps * k0) * LDM;
+                            double* row1 = Mt + (warp + nwarps * k1) * LDM;
+                            const double l0 = __shfl_sync(kFull, lmul, k0), l1 = __shfl_sync(kFull, lmul, k1);
+                            if (k1 != k0) {
+                                for (int j = c + 1 + lane; j < N2 + 3; j += 32) {
+                                    const double p = prow[j], v0 = row0[j], v1 = row1[j];
+                                    row0[j] = v0 - l0 * p;
+                                    row1[j] = v1 - l1 * p;
+                                }
+                            } else {
+                                for (int j = c + 1 + lane; j < N2 + 3; j += 32) row0[j] -= l0 * prow[j];
                             }
-                            __syncwarp();
-                            if (ract && c + 1 < N2) {
-                                const long long key = (long long)abs_bits(Mt[rl * LDM + c + 1]);
-                                if (key > bkey && key <= (long long)kInfBits) { bkey = key; brow = rl; }
-                            }
+                        }
+                        __syncwarp();
+                        long long bkey = -1;   // |entry| bits of this lane's row (-1: none)
+                        const int brow = rl;
+                        if (ract && c + 1 < N2) {
+                            const long long key = (long long)abs_bits(Mt[rl * LDM + c + 1]);
+                            if (key <= (long long)kInfBits) bkey = key;
                         }
                         long long wkey = bkey;
                         for (int off = 16; off > 0; off >>= 1) {
@@ -451,18 +460,28 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                         if (NMC_IN_BOUNDS(g.dbg, i, 128, kDbgHistory)) nd->dinv[i] = 1.0 / Mt[nd->prow[i] * LDM + i];
                     __syncthreads();
                     for (int k = warp; k < 3; k += nwarps) {
+                        // unknown r in lane r % 32's register r / 32, with its row
                         const int col = N2 + k;
-                        for (int i = N2 - 1; i >= 0; --i) {
-                            const int pi = nd->prow[i];
-                            const double xi = Mt[pi * LDM + col] * nd->dinv[i];
-                            __syncwarp();
-                            for (int r = lane; r < i; r += 32) {
-                                const int pr = nd->prow[r];
-                                Mt[pr * LDM + col] -= Mt[pr * LDM + i] * xi;
-                            }
-                            if (lane == 0) Mt[pi * LDM + col] = xi;
-                            __syncwarp();
+                        double y[4];
+                        const double* row[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            row[u] = Mt + nd->prow[min(lane + 32 * u, N2 - 1)] * LDM;
+                            y[u] = lane + 32 * u < N2 ? row[u][col] : 0.0;
                         }
+#pragma unroll
+                        for (int ui = 3; ui >= 0; --ui)
+                            for (int i = min(N2, 32 * ui + 32) - 1; i >= 32 * ui; --i) {
+                                const double xi = __shfl_sync(kFull, y[ui], i & 31) * nd->dinv[i];
+                                if (lane == (i & 31)) y[ui] = xi;
+#pragma unroll
+                                for (int u = 0; u <= ui; ++u)
+                                    if (lane + 32 * u < i) y[u] -= row[u][i] * xi;
+                            }
+                        __syncwarp();
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (lane + 32 * u < N2) Mt[nd->prow[lane + 32 * u] * LDM + col] = y[u];
                     }
                     __syncthreads();
                     if (mine) {   // unknown c sits in its pivot row
@@ -585,7 +604,7 @@ static int launch_adj_impl(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream) {
 
 int launch_adjoint(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream) {
     const int threads = ((ctx->ns * ctx->nep + 31) / 32) * 32;
-    if (threads <= 128) return launch_adj_impl<128, 4>(ctx, a, stream);
+    if (threads <= 128) return launch_adj_impl<128, 2>(ctx, a, stream);
     if (threads <= 256) return launch_adj_impl<256, 2>(ctx, a, stream);
     return launch_adj_impl<512, 1>(ctx, a, stream);
 }
