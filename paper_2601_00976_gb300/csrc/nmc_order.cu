@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kThreads) order_kernel(int n, const double* __
     atomicMax(&top, mx);
     __syncthreads();
     const int k0 = top;
-    for (int i = t; i < n; i += kThreads) atomicAdd(&first[min(k0 - key_of(rho[i], dt[i]), kKeys - 1)], 1);
+    for (int i = t; i < n; i += kThreads) atomicAdd(&first[min(max(k0 - key_of(rho[i], dt[i]), 0), kKeys - 1)], 1);
     __syncthreads();
     for (int off = 1; off < kKeys; off <<= 1) {   // inclusive prefix sums
         const int v = t >= off && t < kKeys ? first[t - off] : 0;
@@ -60,7 +60,9 @@ __global__ void __launch_bounds__(kThreads) order_kernel(int n, const double* __
     __syncthreads();
     if (t < kKeys) first[t] = before;
     __syncthreads();
-    for (int i = t; i < n; i += kThreads) order[atomicAdd(&first[min(k0 - key_of(rho[i], dt[i]), kKeys - 1)], 1)] = i;
+    // the bounds matter only if a caller overwrites rho or dt meanwhile: the passes then disagree
+    for (int i = t; i < n; i += kThreads)
+        order[min(atomicAdd(&first[min(max(k0 - key_of(rho[i], dt[i]), 0), kKeys - 1)], 1), n - 1)] = i;
 }
 
 }  // namespace
