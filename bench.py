@@ -74,10 +74,10 @@ WORKLOAD = ("perturbed collapse profile (+-10% seeded perturbations of rho, T, Y
 # DRAM bytes (read + write) per node of one launch, from ncu captures (dram__bytes_read.sum +
 # dram__bytes_write.sum); traffic grows with the node count.  None where the kernel has changed since its
 # counters were taken.
-TRAFFIC_PER_NODE = {"fused_kernel<double>": 15540.0, "fused_kernel<float>": 14506.0,
-                    "adjoint_kernel": 12079.0, "velocity_kernel": 6029.0,
-                    "c2p_kernel": 530723584 / 65536, "opacity_interp_kernel": 159e6 / (1 << 22),
-                    "opacity_interp_mixed_kernel": 162e6 / (1 << 22)}
+TRAFFIC_PER_NODE = {"fused_kernel<double>": 14829.0, "fused_kernel<float>": 14197.0,
+                    "adjoint_kernel": 12015.0, "velocity_kernel": 5951.0,
+                    "c2p_kernel": 523596032 / 65536, "opacity_interp_fixed_kernel": 169922560 / (1 << 22),
+                    "opacity_interp_mixed_kernel": 168829696 / (1 << 22)}
 
 
 def _traffic(kernel, n):
@@ -569,7 +569,7 @@ def time_c2p(args, ctx, eps, dev, rank, barrier, allmax, stream):
 def time_interp(args, ctx, eps, dev, rank, barrier, allmax, stream):
     """Time opacity_interp (FP64): chi_EmAb and sigma_Iso of every species at scattered points."""
     import torch
-    from paper_2601_00976_gb300 import synthetic, flops
+    from paper_2601_00976_gb300 import synthetic
     from paper_2601_00976_gb300.dist import workload_seed, weak_scaling_value
     P = args.interp_points
     ws = int(os.environ.get("WORLD_SIZE", "1"))
@@ -621,8 +621,6 @@ def time_interp(args, ctx, eps, dev, rank, barrier, allmax, stream):
                           "kernel": "opacity_interp_mixed_kernel",
                           "peak_source": "measured copy bandwidth (MEASURED_PEAKS.json)",
                           "algorithmic_bytes_per_launch": INTERP_BYTES_PER_POINT * P, "kernel_ms": launch_mm}}
-    fl = flops.interp_point_flops() * P
-    ach = fl / (launch_ms * 1e-3) / 1e12
     gbs = INTERP_BYTES_PER_POINT * P / (launch_ms * 1e-3) / 1e9
     return {"metric": "interpolated opacities/s (points*launches*steps/s)",
             "value": weak_scaling_value(ws * P * len(launches), steps, total_ms), "unit": "points/s",
@@ -630,7 +628,11 @@ def time_interp(args, ctx, eps, dev, rank, barrier, allmax, stream):
             "config": {"workload": INTERP_WORKLOAD, "points_per_gpu": P, "launches_per_step": len(launches),
                        "all_values_finite_positive": finite,
                        "hbm_gbs_algorithmic": gbs, "hbm_frac_of_measured": gbs / HBM_PEAK_GBS},
-            "roofline": _fp64_roof(ach, "opacity_interp_kernel", P, fl, launch_ms),
+            "roofline": {"bound": "hbm", "achieved": gbs, "peak": HBM_PEAK_GBS, "unit": "GB/s",
+                         "frac": gbs / HBM_PEAK_GBS, "traffic": _traffic("opacity_interp_fixed_kernel", P),
+                         "kernel": "opacity_interp_fixed_kernel",
+                         "peak_source": "measured copy bandwidth (MEASURED_PEAKS.json); the arithmetic runs in integers",
+                         "algorithmic_bytes_per_launch": INTERP_BYTES_PER_POINT * P, "kernel_ms": launch_ms},
             "mixed": mixed}
 
 

@@ -33,7 +33,8 @@
  *   context.  Numerical trouble at a node is never an error return: it is
  *   reported in that node's status bits.
  * - One context may be used by one stream at a time: calls that overlap in
- *   time on different streams share the context's work-queue counter and race.
+ *   time on different streams share the context's work-queue counter and node
+ *   order and race.
  */
 #ifndef NMC_H
 #define NMC_H
