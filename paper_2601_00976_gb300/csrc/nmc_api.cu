@@ -365,7 +365,6 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
     t.n_quad = (long long)ns * tb->n_ye * (tb->n_t - 1) * (tb->n_rho - 1) * (ne - 1);
     if (rc == NMC_OK) rc = build_f32_cells(ctx, t.emab_f, &t.emab_q);
     if (rc == NMC_OK) rc = build_f32_cells(ctx, t.iso_f, &t.iso_q);
-    if (rc == NMC_OK) rc = build_interp_tables(ctx, tb);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->nes, n_nes, kCW, &t.nes_f);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->pair, n_pair, kCW, &t.pair_f);
     if (rc == NMC_OK) {
@@ -373,12 +372,6 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         e = cudaMalloc(&p, 256);
         if (e != cudaSuccess) rc = NMC_ENOMEM;
         else { ctx->allocations.push_back(p); ctx->queue = static_cast<int*>(p); }
-    }
-    if (rc == NMC_OK) {
-        void* p = nullptr;
-        e = cudaMalloc(&p, kOrderMax * sizeof(int));
-        if (e != cudaSuccess) rc = NMC_ENOMEM;
-        else { ctx->allocations.push_back(p); ctx->order = static_cast<int*>(p); }
     }
 #ifdef NMC_DEBUG
     if (rc == NMC_OK) {   // the bounds-check error word, cleared
@@ -407,11 +400,24 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         if (e == cudaSuccess) e = preload_fused_f32_m3();
         if (e == cudaSuccess) e = preload_fused_f32_m5();
         if (e == cudaSuccess) e = preload_order();
+        // which opacity_interp kernel a call takes depends on its size: none is first loaded under a capture
+        if (e == cudaSuccess) e = preload_interp();
         if (e != cudaSuccess) rc = NMC_ECUDA;
     }
     if (rc == NMC_OK) {
         int* scratch = nullptr;
         rc = noalloc_scratch_address(ctx, &scratch);
+    }
+    // last: optional, and must not take the memory the allocations above need
+    if (rc == NMC_OK) {
+        void* p = nullptr;
+        if (cudaMalloc(&p, kOrderMax * sizeof(int)) == cudaSuccess) {
+            ctx->allocations.push_back(p);
+            ctx->order = static_cast<int*>(p);
+        } else {
+            cudaGetLastError();
+        }
+        rc = build_interp_tables(ctx, tb);
     }
     if (rc != NMC_OK) { nmc_destroy(ctx); return rc; }
     *out = ctx;

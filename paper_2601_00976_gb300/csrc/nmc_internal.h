@@ -263,6 +263,7 @@ int launch_opacity_interp(nmc_ctx* ctx, int which, int species, long long p, con
                           const double* T, const double* Ye, const double* E, double* out,
                           cudaStream_t stream);
 int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb);
+cudaError_t preload_interp();
 int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev);
 int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                                 const double* T, const double* Ye, const double* E, double* out,

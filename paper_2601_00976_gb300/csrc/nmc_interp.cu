@@ -361,6 +361,16 @@ int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev) {
     return NMC_OK;
 }
 
+cudaError_t preload_interp() {
+    cudaFuncAttributes fa;
+    for (const void* k : {(const void*)opacity_interp_kernel, (const void*)opacity_interp_fixed_kernel,
+                          (const void*)opacity_interp_mixed_kernel<1>, (const void*)opacity_interp_mixed_kernel<2>}) {
+        const cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     InterpTables& fx = ctx->fx;
     fx.quads[0] = fx.quads[1] = nullptr;
@@ -386,20 +396,18 @@ int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     if (rc == NMC_OK) rc = upload_fx(ctx, lne.data(), lne.size(), &fx.lne);
     if (rc == NMC_OK) rc = upload_fx(ctx, rec.data(), rec.size(), &fx.rec);
     if (rc == NMC_OK) rc = upload_fx(ctx, sh.data(), sh.size(), &fx.sh);
-    if (rc != NMC_OK) return rc;
+    if (rc != NMC_OK) return rc == NMC_ENOMEM ? NMC_OK : rc;   // too little memory: the FP64 form serves
     const long long nrows = (long long)ctx->ns * tb->n_ye * tb->n_t;
-    const size_t bytes = (size_t)nrows * (tb->n_rho - 1) * (ne - 1) * 32;
-    ulonglong2* q[2] = {nullptr, nullptr};
-    for (int w = 0; w < 2; ++w) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {   // too little memory for the cells: the FP64 form serves
-            cudaGetLastError();
-            return NMC_OK;
-        }
-        ctx->allocations.push_back(p);
-        q[w] = static_cast<ulonglong2*>(p);
-        fixed_quads_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? ctx->tb.emab : ctx->tb.iso, nrows, tb->n_rho, ne, q[w]);
+    const size_t cells = (size_t)nrows * (tb->n_rho - 1) * (ne - 1) * 2;   // of one table, in ulonglong2
+    void* p = nullptr;
+    if (cudaMalloc(&p, 2 * cells * sizeof(ulonglong2)) != cudaSuccess) {
+        cudaGetLastError();
+        return NMC_OK;
     }
+    ctx->allocations.push_back(p);
+    ulonglong2* const q[2] = {static_cast<ulonglong2*>(p), static_cast<ulonglong2*>(p) + cells};
+    for (int w = 0; w < 2; ++w)
+        fixed_quads_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? ctx->tb.emab : ctx->tb.iso, nrows, tb->n_rho, ne, q[w]);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("fixed-point tables: ") + cudaGetErrorString(e));

@@ -94,3 +94,20 @@ def test_points_do_not_depend_on_the_batch(n):
             part = ctx.opacity_interp(1, 1, *[p[i:i + 2000].contiguous() for p in pts], mixed=mixed)
             assert torch.equal(part, whole[i:i + 2000])
     ctx.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("n", [1000, 700001])
+def test_first_call_under_capture(n, mixed):
+    """A context's first interpolation, recorded in a graph, gives the eager call's bits (either batch size's kernel)."""
+    edges, g, tables, _ = make_case(10, 3.0, 2, 2, "profile", 1)
+    ctx = nmc.Context(edges, 2, 2, tables)
+    pts = [p.contiguous() for p in _points(np.random.default_rng(7), g, n)]
+    out = torch.zeros(n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.opacity_interp(0, 1, *pts, out=out, mixed=mixed)
+    graph.replay()
+    assert torch.equal(out, ctx.opacity_interp(0, 1, *pts, mixed=mixed))
+    ctx.close()
