@@ -157,8 +157,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
 #endif
     for (;;) {
         if (tid == 0) {
-            long long nn = atomicAdd(a.queue, 1);
-            if (a.order && nn < a.n) nn = a.order[nn];
+            long long nn = node_at(a.order, atomicAdd(a.queue, 1), a.n);
 #ifdef NMC_DEBUG
             if (g.dbg && *reinterpret_cast<volatile unsigned*>(g.dbg) != 0u) nn = a.n;   // a check failed: stop
 #endif

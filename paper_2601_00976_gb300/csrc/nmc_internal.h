@@ -273,6 +273,14 @@ int launch_adjoint(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream);
 int launch_plain(nmc_ctx* ctx, const SolveArgs& a, cudaStream_t stream);
 // Clears the work queue of a launch with `resident` blocks and, where it pays, orders the nodes (a.order stays set)
 constexpr int kOrderMax = 1 << 16;
+// The k-th node of a launch of n (order null: nodes in index order).  An entry of the order may belong to another
+// batch, or to none, when a caller breaks the one-stream rule or overwrites rho or dt while the call runs: it is
+// held to the batch, so that no block leaves the inputs or ends early with nodes left.
+__host__ __device__ __forceinline__ long long node_at(const int* order, long long k, long long n) {
+    if (!order || k >= n) return k;
+    const long long v = order[k];
+    return v < 0 ? 0 : (v >= n ? n - 1 : v);
+}
 int start_queue(nmc_ctx* ctx, SolveArgs& a, long long resident, cudaStream_t stream);
 cudaError_t preload_order();
 int launch_velocity(nmc_ctx* ctx, const SolveArgs& a, const double* v_in, double* v_out, int freeze,

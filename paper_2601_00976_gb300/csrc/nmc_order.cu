@@ -60,7 +60,8 @@ __global__ void __launch_bounds__(kThreads) order_kernel(int n, const double* __
     __syncthreads();
     if (t < kKeys) first[t] = before;
     __syncthreads();
-    // the bounds matter only if a caller overwrites rho or dt meanwhile: the passes then disagree
+    // the bounds matter only if a caller overwrites rho or dt meanwhile: the passes then disagree, and some
+    // entries keep an earlier batch's nodes or are written twice (node_at bounds what is read)
     for (int i = t; i < n; i += kThreads)
         order[min(atomicAdd(&first[min(max(k0 - key_of(rho[i], dt[i]), 0), kKeys - 1)], 1), n - 1)] = i;
 }

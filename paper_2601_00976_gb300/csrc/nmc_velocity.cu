@@ -216,10 +216,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
         for (int c = 0; c < 4; ++c) { Fh[j][c] = 0.0; Qh[j][c] = 0.0; }
 
     for (;;) {
-        if (tid == 0) {
-            const int nn = atomicAdd(a.queue, 1);
-            nd->node = a.order && nn < a.n ? a.order[nn] : nn;
-        }
+        if (tid == 0) nd->node = node_at(a.order, atomicAdd(a.queue, 1), a.n);
         __syncthreads();
         const long long n = nd->node;
         if (n >= a.n) break;
