@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -14,6 +15,21 @@ namespace nmc {
 int set_error(nmc_ctx* ctx, int code, const std::string& msg) {
     if (ctx) ctx->last_error = msg;
     return code;
+}
+
+int device_alloc(nmc_ctx* ctx, size_t bytes, void** p) {
+    *p = nullptr;
+#ifdef NMC_DEBUG
+    if (ctx->fail_alloc > 0 && --ctx->fail_alloc == 0) bytes = size_t(1) << 60;   // no device has as much
+#endif
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();   // told here: left pending, it would come back as the next launch's error
+        *p = nullptr;
+        return set_error(ctx, NMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
+    ctx->allocations.push_back(*p);
+    return NMC_OK;
 }
 
 namespace {
@@ -85,10 +101,9 @@ bool invert_small(std::vector<double>& A, int n) {   // Gauss--Jordan, row-major
 template <typename T>
 int upload(nmc_ctx* ctx, const T* host, size_t count, const T** dev) {
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, count * sizeof(T));
-    if (e != cudaSuccess) return set_error(ctx, NMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    ctx->allocations.push_back(p);
-    e = cudaMemcpy(p, host, count * sizeof(T), cudaMemcpyHostToDevice);
+    const int rc = device_alloc(ctx, count * sizeof(T), &p);
+    if (rc != NMC_OK) return rc;
+    const cudaError_t e = cudaMemcpy(p, host, count * sizeof(T), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));
     *dev = static_cast<const T*>(p);
     return NMC_OK;
@@ -243,6 +258,9 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
     ctx->nep = nep;
     if (ns * nep > 1024) { delete ctx; return NMC_EUNSUPPORTED; }
 
+#ifdef NMC_DEBUG
+    if (const char* k = std::getenv("NMC_FAIL_ALLOC")) ctx->fail_alloc = std::atoi(k);
+#endif
     cudaError_t e = cudaGetDevice(&ctx->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
@@ -369,26 +387,23 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->pair, n_pair, kCW, &t.pair_f);
     if (rc == NMC_OK) {
         void* p = nullptr;
-        e = cudaMalloc(&p, 256);
-        if (e != cudaSuccess) rc = NMC_ENOMEM;
-        else { ctx->allocations.push_back(p); ctx->queue = static_cast<int*>(p); }
+        rc = device_alloc(ctx, 256, &p);
+        ctx->queue = static_cast<int*>(p);
     }
 #ifdef NMC_DEBUG
     if (rc == NMC_OK) {   // the bounds-check error word, cleared
         void* p = nullptr;
-        e = cudaMalloc(&p, 256);
-        if (e == cudaSuccess) e = cudaMemset(p, 0, 256);
-        if (e != cudaSuccess) rc = NMC_ENOMEM;
-        else { ctx->allocations.push_back(p); ctx->g.dbg = static_cast<unsigned*>(p); }
+        rc = device_alloc(ctx, 256, &p);
+        if (rc == NMC_OK && cudaMemset(p, 0, 256) != cudaSuccess) rc = NMC_ECUDA;
+        ctx->g.dbg = static_cast<unsigned*>(p);
     }
 #endif
 #ifdef NMC_TRACE
     if (rc == NMC_OK) {   // the stage counters, cleared
         void* p = nullptr;
-        e = cudaMalloc(&p, kTraceWords * sizeof(unsigned long long));
-        if (e == cudaSuccess) e = cudaMemset(p, 0, kTraceWords * sizeof(unsigned long long));
-        if (e != cudaSuccess) rc = NMC_ENOMEM;
-        else { ctx->allocations.push_back(p); ctx->g.trace = static_cast<unsigned long long*>(p); }
+        rc = device_alloc(ctx, kTraceWords * sizeof(unsigned long long), &p);
+        if (rc == NMC_OK && cudaMemset(p, 0, kTraceWords * sizeof(unsigned long long)) != cudaSuccess) rc = NMC_ECUDA;
+        ctx->g.trace = static_cast<unsigned long long*>(p);
     }
 #endif
     // Set-up of collision_solve_noalloc, done here because this call may allocate: load the fused
@@ -411,13 +426,10 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
     // last: optional, and must not take the memory the allocations above need
     if (rc == NMC_OK) {
         void* p = nullptr;
-        if (cudaMalloc(&p, kOrderMax * sizeof(int)) == cudaSuccess) {
-            ctx->allocations.push_back(p);
-            ctx->order = static_cast<int*>(p);
-        } else {
-            cudaGetLastError();
-        }
+        device_alloc(ctx, kOrderMax * sizeof(int), &p);
+        ctx->order = static_cast<int*>(p);
         rc = build_interp_tables(ctx, tb);
+        if (rc == NMC_OK) ctx->last_error.clear();
     }
     if (rc != NMC_OK) { nmc_destroy(ctx); return rc; }
     *out = ctx;

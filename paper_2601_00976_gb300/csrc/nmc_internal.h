@@ -250,6 +250,9 @@ struct nmc_ctx {
     nmc::HostPipe host_pipe;
     // autotuned fused-kernel variants, keyed by precision, Anderson depth and block class
     std::map<int, nmc::FusedVariant> tuned;
+#ifdef NMC_DEBUG
+    int fail_alloc = 0;   // NMC_FAIL_ALLOC: which device_alloc of the context is to fail (0: none)
+#endif
     int device = 0;
     int num_sms = 0;
     int max_smem_optin = 0;
@@ -300,6 +303,8 @@ int noalloc_scratch_address(nmc_ctx* ctx, int** out);
 int autotune_fused(nmc_ctx* ctx, const SolveArgs& a, cudaStream_t stream, int32_t* chosen, float* chosen_ms);
 size_t adjoint_smem_bytes(const nmc_ctx* ctx, AdjointArgs* a);
 int set_error(nmc_ctx* ctx, int code, const std::string& msg);
+// Device memory that lives as long as the context; NMC_ENOMEM, with *p null, if there is too little.
+int device_alloc(nmc_ctx* ctx, size_t bytes, void** p);
 void host_pipe_release(nmc_ctx* ctx);
 }  // namespace nmc
 

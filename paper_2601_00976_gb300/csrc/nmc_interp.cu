@@ -243,10 +243,9 @@ bool fixed_axis(double lo, double hi, int n, FixedAxis* ax) {
 template <typename T>
 int upload_fx(nmc_ctx* ctx, const T* host, size_t count, const T** dev) {
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, count * sizeof(T));
-    if (e != cudaSuccess) return set_error(ctx, NMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    ctx->allocations.push_back(p);
-    e = cudaMemcpy(p, host, count * sizeof(T), cudaMemcpyHostToDevice);
+    const int rc = device_alloc(ctx, count * sizeof(T), &p);
+    if (rc != NMC_OK) return rc;
+    const cudaError_t e = cudaMemcpy(p, host, count * sizeof(T), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));
     *dev = static_cast<const T*>(p);
     return NMC_OK;
@@ -350,11 +349,10 @@ int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev) {
     const DevTables& t = ctx->tb;
     const long long nsy = (long long)ctx->ns * t.ye.n;
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, (size_t)t.n_quad * 2 * sizeof(float4));
-    if (e != cudaSuccess) return set_error(ctx, NMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    ctx->allocations.push_back(p);
+    const int rc = device_alloc(ctx, (size_t)t.n_quad * 2 * sizeof(float4), &p);
+    if (rc != NMC_OK) return rc;
     f32_cells_kernel<<<ctx->num_sms * 8, 256>>>(tab, nsy, t.t.n, t.rho.n, ctx->ne, static_cast<float4*>(p));
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("FP32 cells: ") + cudaGetErrorString(e));
     *dev = static_cast<const float4*>(p);
@@ -400,11 +398,7 @@ int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     const long long nrows = (long long)ctx->ns * tb->n_ye * tb->n_t;
     const size_t cells = (size_t)nrows * (tb->n_rho - 1) * (ne - 1) * 2;   // of one table, in ulonglong2
     void* p = nullptr;
-    if (cudaMalloc(&p, 2 * cells * sizeof(ulonglong2)) != cudaSuccess) {
-        cudaGetLastError();
-        return NMC_OK;
-    }
-    ctx->allocations.push_back(p);
+    if (device_alloc(ctx, 2 * cells * sizeof(ulonglong2), &p) != NMC_OK) return NMC_OK;
     ulonglong2* const q[2] = {static_cast<ulonglong2*>(p), static_cast<ulonglong2*>(p) + cells};
     for (int w = 0; w < 2; ++w)
         fixed_quads_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? ctx->tb.emab : ctx->tb.iso, nrows, tb->n_rho, ne, q[w]);
