@@ -170,6 +170,10 @@ void nmc_default_params(nmc_params* p);
  * per-block shared-memory footprint <= 227 KB (FP64: ne <= 64 with 4 species).
  * On success *out owns all device memory it allocated; free it with
  * nmc_destroy.  On failure *out is NULL and the return code says why.
+ * A context needs device memory for its tables in FP64 and FP32.  Two
+ * rearranged copies of emab and iso, each four times their FP64 size, only make
+ * opacity_interp and opacity_interp_mixed faster: each is made when it takes no
+ * more than an eighth of the memory then free, and done without otherwise.
  */
 int nmc_create(const nmc_grid* grid, const nmc_tables* tables, nmc_ctx** out);
 

@@ -32,6 +32,13 @@ int device_alloc(nmc_ctx* ctx, size_t bytes, void** p) {
     return NMC_OK;
 }
 
+int spare_alloc(nmc_ctx* ctx, size_t bytes, void** p) {
+    *p = nullptr;
+    size_t left = 0, total = 0;
+    if (cudaMemGetInfo(&left, &total) != cudaSuccess) cudaGetLastError();
+    return bytes <= left / 8 ? device_alloc(ctx, bytes, p) : NMC_ENOMEM;
+}
+
 namespace {
 
 // N-point Gauss--Legendre rule on (-1/2, 1/2) with weights summing to one
@@ -380,9 +387,6 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
     // FP32 copies for the mixed path; kernel tables prescaled by 4 pi / (hc)^3
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->emab, n_op, 1.0, &t.emab_f);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->iso, n_op, 1.0, &t.iso_f);
-    t.n_quad = (long long)ns * tb->n_ye * (tb->n_t - 1) * (tb->n_rho - 1) * (ne - 1);
-    if (rc == NMC_OK) rc = build_f32_cells(ctx, t.emab_f, &t.emab_q);
-    if (rc == NMC_OK) rc = build_f32_cells(ctx, t.iso_f, &t.iso_q);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->nes, n_nes, kCW, &t.nes_f);
     if (rc == NMC_OK) rc = upload_f32(ctx, tb->pair, n_pair, kCW, &t.pair_f);
     if (rc == NMC_OK) {
@@ -423,12 +427,15 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         int* scratch = nullptr;
         rc = noalloc_scratch_address(ctx, &scratch);
     }
-    // last: optional, and must not take the memory the allocations above need
+    // Last: optional, and must not take the memory the allocations above need.  The lookups' cells are four
+    // times the FP64 ln tables each (4 species, 32 energies: 122 and 126 MB); without them the lookups read the
+    // tables themselves.
     if (rc == NMC_OK) {
         void* p = nullptr;
         device_alloc(ctx, kOrderMax * sizeof(int), &p);
         ctx->order = static_cast<int*>(p);
-        rc = build_interp_tables(ctx, tb);
+        rc = build_f32_cells(ctx);
+        if (rc == NMC_OK) rc = build_interp_tables(ctx, tb);
         if (rc == NMC_OK) ctx->last_error.clear();
     }
     if (rc != NMC_OK) { nmc_destroy(ctx); return rc; }

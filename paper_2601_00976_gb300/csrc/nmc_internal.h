@@ -130,7 +130,7 @@ struct DevTables {
     long long n_op, n_nes, n_pair;   // element counts of the EmAb/Iso, NES and pair tables
     // opacity_interp_mixed: the FP32 ln tables regrouped per (T, rho, E) cell, two float4
     // (rho_i E_q, rho_i+1 E_q, rho_i E_q+1, rho_i+1 E_q+1) at T_j and T_j+1 per
-    // [ns][nye][nt-1][nrho-1][ne-1]; n_quad cells
+    // [ns][nye][nt-1][nrho-1][ne-1]; n_quad cells.  Both null where memory is short (build_f32_cells)
     const float4* emab_q;
     const float4* iso_q;
     long long n_quad;
@@ -267,7 +267,7 @@ int launch_opacity_interp(nmc_ctx* ctx, int which, int species, long long p, con
                           cudaStream_t stream);
 int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb);
 cudaError_t preload_interp();
-int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev);
+int build_f32_cells(nmc_ctx* ctx);
 int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long p, const double* rho,
                                 const double* T, const double* Ye, const double* E, double* out,
                                 cudaStream_t stream);
@@ -305,6 +305,8 @@ size_t adjoint_smem_bytes(const nmc_ctx* ctx, AdjointArgs* a);
 int set_error(nmc_ctx* ctx, int code, const std::string& msg);
 // Device memory that lives as long as the context; NMC_ENOMEM, with *p null, if there is too little.
 int device_alloc(nmc_ctx* ctx, size_t bytes, void** p);
+// The same for what only makes calls faster: at most an eighth of the memory that is free, the rest is the caller's.
+int spare_alloc(nmc_ctx* ctx, size_t bytes, void** p);
 void host_pipe_release(nmc_ctx* ctx);
 }  // namespace nmc
 

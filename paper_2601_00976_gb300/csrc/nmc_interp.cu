@@ -23,7 +23,9 @@
 // four with (rho, E) cells, which left the kernel at the L2's rate: 8.6 TB/s of
 // sectors for 2.1 TB/s of points), and two points a thread are in flight.
 // 8.4 M points: 0.168 ms before these and the integer conversions, 0.121 ms now
-// (2.8 TB/s of points, 41% of the copy rate).
+// (2.8 TB/s of points, 41% of the copy rate).  A context too short of memory for
+// the cells reads the 16 values from the FP32 tables themselves: the same bits,
+// 0.29 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -261,8 +263,8 @@ __device__ __forceinline__ void cell_f(float v, const Axis& ax, int* i, float* t
     *t = x - (float)c;
 }
 
-// U points per thread and step, kPointStride apart, so that their loads are in flight together.
-template <int U>
+// U points per thread and step, so that their loads are in flight together; kCells: see the file's head.
+template <int U, bool kCells>
 __global__ void __launch_bounds__(kBuckets) opacity_interp_mixed_kernel(const DevGrid g, const DevTables tb, int which,
                                                                         int species, long long p,
                                                                         const double* __restrict__ rho,
@@ -279,8 +281,9 @@ __global__ void __launch_bounds__(kBuckets) opacity_interp_mixed_kernel(const De
     lut[threadIdx.x] = (unsigned char)cell_by_bisection(lne, NE, lo_e + ((int)threadIdx.x - 1) * per_bucket);
     __syncthreads();
     const float4* __restrict__ tab = which == 0 ? tb.emab_q : tb.iso_q;
-    const int nrc = tb.rho.n - 1, nec = NE - 1, ntc = tb.t.n - 1;
-    const long long dY = (long long)ntc * nrc * nec, sp0 = (long long)species * tb.ye.n;
+    const float* __restrict__ row = which == 0 ? tb.emab_f : tb.iso_f;
+    const int nt = kCells ? tb.t.n - 1 : tb.t.n, nr = kCells ? tb.rho.n - 1 : tb.rho.n, ne = kCells ? NE - 1 : NE;
+    const long long dT = (long long)nr * ne, dY = nt * dT, sp0 = (long long)species * tb.ye.n;
     const long long step = (long long)gridDim.x * blockDim.x;
     for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < p; i0 += U * step) {
         float fr[U], ft[U], fy[U], fe[U];
@@ -307,11 +310,20 @@ __global__ void __launch_bounds__(kBuckets) opacity_interp_mixed_kernel(const De
             const int lo = cell_from(lne, NE, le, (int)lut[b < kBuckets ? b : kBuckets - 1]);
             te[u] = (le - lne[lo]) / (lne[lo + 1] - lne[lo]);
             // the (T, rho, E) cell's eight corners are one 32-byte sector; (T, Ye) corners k = cb + 2 cc
-            const long long base = (((sp0 + iy) * ntc + it) * nrc + ir) * nec + lo;
-            const bool ok = NMC_IN_BOUNDS(g.dbg, base, tb.n_quad, kDbgEmabIso) &&
-                            NMC_IN_BOUNDS(g.dbg, base + dY, tb.n_quad, kDbgEmabIso);
+            const long long base = (((sp0 + iy) * nt + it) * nr + ir) * ne + lo;
+            const bool ok = NMC_IN_BOUNDS(g.dbg, base, kCells ? tb.n_quad : tb.n_op, kDbgEmabIso) &&
+                            NMC_IN_BOUNDS(g.dbg, base + dY + (kCells ? 0 : dT + ne + 1), kCells ? tb.n_quad : tb.n_op, kDbgEmabIso);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) c[u][k] = ok ? __ldg(tab + 2 * (base + (k >> 1) * dY) + (k & 1)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k < 4; ++k) {
+                c[u][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (!ok) continue;
+                if constexpr (kCells) {
+                    c[u][k] = __ldg(tab + 2 * (base + (k >> 1) * dY) + (k & 1));
+                } else {
+                    const float* r0 = row + base + (k & 1) * dT + (k >> 1) * dY;
+                    c[u][k] = make_float4(__ldg(r0), __ldg(r0 + ne), __ldg(r0 + 1), __ldg(r0 + ne + 1));
+                }
+            }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -345,24 +357,31 @@ __global__ void f32_cells_kernel(const float* __restrict__ tab, long long nsy, i
 
 }  // namespace
 
-int build_f32_cells(nmc_ctx* ctx, const float* tab, const float4** dev) {
-    const DevTables& t = ctx->tb;
+int build_f32_cells(nmc_ctx* ctx) {
+    DevTables& t = ctx->tb;
     const long long nsy = (long long)ctx->ns * t.ye.n;
+    t.emab_q = t.iso_q = nullptr;
+    t.n_quad = nsy * (t.t.n - 1) * (t.rho.n - 1) * (ctx->ne - 1);
+    const size_t cells = (size_t)t.n_quad * 2;   // of one table, in float4
     void* p = nullptr;
-    const int rc = device_alloc(ctx, (size_t)t.n_quad * 2 * sizeof(float4), &p);
-    if (rc != NMC_OK) return rc;
-    f32_cells_kernel<<<ctx->num_sms * 8, 256>>>(tab, nsy, t.t.n, t.rho.n, ctx->ne, static_cast<float4*>(p));
+    if (spare_alloc(ctx, 2 * cells * sizeof(float4), &p) != NMC_OK) return NMC_OK;
+    float4* const q[2] = {static_cast<float4*>(p), static_cast<float4*>(p) + cells};
+    for (int w = 0; w < 2; ++w)
+        f32_cells_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? t.emab_f : t.iso_f, nsy, t.t.n, t.rho.n, ctx->ne, q[w]);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("FP32 cells: ") + cudaGetErrorString(e));
-    *dev = static_cast<const float4*>(p);
+    t.emab_q = q[0];
+    t.iso_q = q[1];
     return NMC_OK;
 }
 
 cudaError_t preload_interp() {
     cudaFuncAttributes fa;
     for (const void* k : {(const void*)opacity_interp_kernel, (const void*)opacity_interp_fixed_kernel,
-                          (const void*)opacity_interp_mixed_kernel<1>, (const void*)opacity_interp_mixed_kernel<2>}) {
+                          (const void*)opacity_interp_mixed_kernel<1, true>,
+                          (const void*)opacity_interp_mixed_kernel<2, true>,
+                          (const void*)opacity_interp_mixed_kernel<1, false>}) {
         const cudaError_t e = cudaFuncGetAttributes(&fa, k);
         if (e != cudaSuccess) return e;
     }
@@ -398,7 +417,7 @@ int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     const long long nrows = (long long)ctx->ns * tb->n_ye * tb->n_t;
     const size_t cells = (size_t)nrows * (tb->n_rho - 1) * (ne - 1) * 2;   // of one table, in ulonglong2
     void* p = nullptr;
-    if (device_alloc(ctx, 2 * cells * sizeof(ulonglong2), &p) != NMC_OK) return NMC_OK;
+    if (spare_alloc(ctx, 2 * cells * sizeof(ulonglong2), &p) != NMC_OK) return NMC_OK;
     ulonglong2* const q[2] = {static_cast<ulonglong2*>(p), static_cast<ulonglong2*>(p) + cells};
     for (int w = 0; w < 2; ++w)
         fixed_quads_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? ctx->tb.emab : ctx->tb.iso, nrows, tb->n_rho, ne, q[w]);
@@ -418,11 +437,10 @@ int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long 
     long long blocks = (p + threads - 1) / threads;
     const long long cap = (long long)ctx->num_sms * 8;
     // two points a thread once every SM has its blocks; below that one, so that the points spread over the SMs
-    if (blocks >= 2 * cap)
-        opacity_interp_mixed_kernel<2><<<(unsigned)cap, threads, 0, stream>>>(ctx->g, ctx->tb, which, species, p, rho, T, Ye, E, out);
-    else
-        opacity_interp_mixed_kernel<1><<<(unsigned)(blocks > cap ? cap : blocks), threads, 0, stream>>>(ctx->g, ctx->tb, which,
-                                                                                                  species, p, rho, T, Ye, E, out);
+    const bool cells = ctx->tb.emab_q != nullptr;
+    auto kern = !cells ? opacity_interp_mixed_kernel<1, false>
+                       : (blocks >= 2 * cap ? opacity_interp_mixed_kernel<2, true> : opacity_interp_mixed_kernel<1, true>);
+    kern<<<(unsigned)(blocks > cap ? cap : blocks), threads, 0, stream>>>(ctx->g, ctx->tb, which, species, p, rho, T, Ye, E, out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return set_error(ctx, NMC_ECUDA, std::string("opacity_interp_mixed launch: ") + cudaGetErrorString(e));

@@ -35,9 +35,10 @@ def calls(ctx):
 
 whole = nmc.Context(edges, 1, 2, tables)
 ref = calls(whole)
-refused, served, exact = 0, 0, 0
+refused, served, exact, uses = 0, 0, 0, []
 for k in range(1, 61):
     os.environ["NMC_FAIL_ALLOC"] = str(k)
+    free = torch.cuda.mem_get_info()[0]
     try:
         ctx = nmc.Context(edges, 1, 2, tables)
     except nmc.NmcError as e:
@@ -47,14 +48,19 @@ for k in range(1, 61):
         torch.ones(3, device="cuda").sum().item()
         continue
     assert ctx.last_error() == "", ctx.last_error()
+    used = free - torch.cuda.mem_get_info()[0]
     got = calls(ctx)
     assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
     assert torch.max(torch.abs(got[2] - ref[2]) / ref[2]).item() <= 1e-13
     served += 1
     exact += int(torch.equal(got[2], ref[2]))
+    uses.append((used, torch.equal(got[2], ref[2])))
     ctx.close()
 del os.environ["NMC_FAIL_ALLOC"]
-print("ALLOC", refused, served, exact)
+# the FP32 lookup's cells, 2 x 2 x 16 x 31 x 31 x 9 of 32 bytes, are one allocation (17.7 MB), the FP64 form's another
+most = max(u for u, _ in uses)
+no_cells = sum(1 for u, same in uses if same and u < most - (14 << 20))
+print("ALLOC", refused, served, exact, no_cells)
 """
 
 
@@ -64,6 +70,7 @@ def test_each_allocation_failing_in_turn():
     env = dict(os.environ, NMC_DEBUG="1")
     r = subprocess.run([sys.executable, "-c", CHILD, ROOT], capture_output=True, text=True, env=env, timeout=900)
     assert r.returncode == 0, r.stderr[-3000:]
-    refused, served, exact = (int(x) for x in r.stdout.split("ALLOC")[1].split())
+    refused, served, exact, no_cells = (int(x) for x in r.stdout.split("ALLOC")[1].split())
     # the required tables, then those that are optional, then a k beyond the last allocation
     assert refused >= 20 and served - exact >= 5 and exact >= 5, (refused, served, exact)
+    assert no_cells == 1, no_cells   # a context without the FP32 lookup's cells was served
