@@ -369,7 +369,7 @@ int build_f32_cells(nmc_ctx* ctx) {
     for (int w = 0; w < 2; ++w)
         f32_cells_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? t.emab_f : t.iso_f, nsy, t.t.n, t.rho.n, ctx->ne, q[w]);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);   // the fill's stream: others may be at work
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("FP32 cells: ") + cudaGetErrorString(e));
     t.emab_q = q[0];
     t.iso_q = q[1];
@@ -422,7 +422,7 @@ int build_interp_tables(nmc_ctx* ctx, const nmc_tables* tb) {
     for (int w = 0; w < 2; ++w)
         fixed_quads_kernel<<<ctx->num_sms * 8, 256>>>(w == 0 ? ctx->tb.emab : ctx->tb.iso, nrows, tb->n_rho, ne, q[w]);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);   // the fill's stream: others may be at work
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("fixed-point tables: ") + cudaGetErrorString(e));
     fx.n_quad = nrows * (tb->n_rho - 1) * (ne - 1);
     fx.quads[0] = q[0];
