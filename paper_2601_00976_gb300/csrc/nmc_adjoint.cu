@@ -579,34 +579,66 @@ size_t adjoint_smem_bytes(const nmc_ctx* ctx, AdjointArgs* a) {
     return b_mats + b_mat + b_vec + b_red + b_node;
 }
 
+// Blocks of the shape that an SM holds, and their shared memory; or an error.
 template <int MAXT, int MINB>
-static int launch_adj_impl(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream) {
+static int adj_resident(nmc_ctx* ctx, AdjointArgs& a, size_t* smem, int* per_sm) {
     auto kern = adjoint_kernel<MAXT, MINB>;
     if (2 * ctx->ne > 128)   // the reciprocal diagonal of a pair system holds 2 ne <= 128 entries
         return set_error(ctx, NMC_EUNSUPPORTED, "collision_adjoint supports at most 64 energies");
-    const size_t smem = adjoint_smem_bytes(ctx, &a);
-    if ((int)smem > ctx->max_smem_optin)
+    *smem = adjoint_smem_bytes(ctx, &a);
+    if ((int)*smem > ctx->max_smem_optin)
         return set_error(ctx, NMC_EUNSUPPORTED, "shared-memory footprint of the adjoint kernel exceeds the per-block limit");
     const int threads = ((ctx->ns * ctx->nep + 31) / 32) * 32;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-    if (e != cudaSuccess || per_sm < 1)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, *smem);
+    if (e != cudaSuccess || *per_sm < 1)
         return set_error(ctx, NMC_EUNSUPPORTED, "adjoint kernel cannot be resident with this shape");
+    return NMC_OK;
+}
+
+template <int MAXT, int MINB>
+static int launch_adj_impl(nmc_ctx* ctx, AdjointArgs& a, size_t smem, int per_sm, cudaStream_t stream) {
+    const int threads = ((ctx->ns * ctx->nep + 31) / 32) * 32;
     long long grid = (long long)per_sm * ctx->num_sms;
     if (grid > a.n) grid = a.n;
-    kern<<<(unsigned)grid, threads, smem, stream>>>(a);
-    e = cudaGetLastError();
+    adjoint_kernel<MAXT, MINB><<<(unsigned)grid, threads, smem, stream>>>(a);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(ctx, NMC_ECUDA, std::string("adjoint kernel launch: ") + cudaGetErrorString(e));
     return NMC_OK;
 }
 
 int launch_adjoint(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream) {
     const int threads = ((ctx->ns * ctx->nep + 31) / 32) * 32;
-    if (threads <= 128) return launch_adj_impl<128, 2>(ctx, a, stream);
-    if (threads <= 256) return launch_adj_impl<256, 2>(ctx, a, stream);
-    return launch_adj_impl<512, 1>(ctx, a, stream);
+    size_t smem = 0;
+    int wide = 0, narrow = 0, rc;
+    if (threads <= 128) {
+        // Two register classes: 231 registers a thread (two 128-thread blocks an SM) and 128 (four).  The wide one
+        // is the faster block (one wave of 300 nodes 3-5% faster at every shape), and the better one where shared
+        // memory or the batch leaves no more blocks than its registers hold: 8192 nodes, 4 species, 32 energies,
+        // 18.0 against 18.7 ms.  Smaller shapes have shared memory for more blocks, which the narrow class lets in: 4
+        // species, 24 energies 13.5 -> 11.4 ms, 20 energies (constant elements) 12.4 -> 10.2, 10 energies 5.3 -> 4.9;
+        // 6 species, 16 energies 10.9 -> 7.8.
+        rc = adj_resident<128, 2>(ctx, a, &smem, &wide);
+        if (rc == NMC_OK && a.n > (long long)wide * ctx->num_sms) rc = adj_resident<128, 4>(ctx, a, &smem, &narrow);
+        if (rc != NMC_OK) return rc;
+        return narrow > wide ? launch_adj_impl<128, 4>(ctx, a, smem, narrow, stream)
+                             : launch_adj_impl<128, 2>(ctx, a, smem, wide, stream);
+    }
+    rc = threads <= 256 ? adj_resident<256, 2>(ctx, a, &smem, &wide) : adj_resident<512, 1>(ctx, a, &smem, &wide);
+    if (rc != NMC_OK) return rc;
+    return threads <= 256 ? launch_adj_impl<256, 2>(ctx, a, smem, wide, stream)
+                          : launch_adj_impl<512, 1>(ctx, a, smem, wide, stream);
+}
+
+cudaError_t preload_adjoint() {
+    cudaFuncAttributes fa;
+    for (const void* k : {(const void*)adjoint_kernel<128, 2>, (const void*)adjoint_kernel<128, 4>,
+                          (const void*)adjoint_kernel<256, 2>, (const void*)adjoint_kernel<512, 1>}) {
+        const cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace nmc

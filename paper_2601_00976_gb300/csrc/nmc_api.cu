@@ -419,8 +419,10 @@ int nmc_create(const nmc_grid* grid, const nmc_tables* tb, nmc_ctx** out) {
         if (e == cudaSuccess) e = preload_fused_f32_m3();
         if (e == cudaSuccess) e = preload_fused_f32_m5();
         if (e == cudaSuccess) e = preload_order();
-        // which opacity_interp kernel a call takes depends on its size: none is first loaded under a capture
+        // which opacity_interp or collision_adjoint kernel a call takes depends on its size: none is first loaded
+        // under a capture
         if (e == cudaSuccess) e = preload_interp();
+        if (e == cudaSuccess) e = preload_adjoint();
         if (e != cudaSuccess) rc = NMC_ECUDA;
     }
     if (rc == NMC_OK) {

@@ -273,6 +273,7 @@ int launch_opacity_interp_mixed(nmc_ctx* ctx, int which, int species, long long 
                                 cudaStream_t stream);
 size_t fused_smem_bytes(const nmc_ctx* ctx, int maxm, bool mixed, SolveArgs* a);
 int launch_adjoint(nmc_ctx* ctx, AdjointArgs& a, cudaStream_t stream);
+cudaError_t preload_adjoint();
 int launch_plain(nmc_ctx* ctx, const SolveArgs& a, cudaStream_t stream);
 // Clears the work queue of a launch with `resident` blocks and, where it pays, orders the nodes (a.order stays set)
 constexpr int kOrderMax = 1 << 16;
