@@ -333,6 +333,10 @@ __device__ __forceinline__ VoteLimit vote_limit(double thr) {
     return l;
 }
 
+// A bin's FP32 weight for the filter below; NaN (no filter: every sum is formed in FP64) where the FP32 value
+// has lost digits or the range, on grids of energies below ~1e-12 or above ~1e12 MeV.
+__device__ __forceinline__ float vote_weight(float w) { return w >= 1.17549435e-38f && w <= 3.4e38f ? w : __int_as_float(0x7fc00000); }
+
 // |x| 2^-e (biased exponent e) truncated to FP32; 0 below its range, infinity above or for NaN
 __device__ __forceinline__ float scaled_abs(double x, int e) {
     const int hi = __double2hiint(x) & 0x7fffffff, ex = (hi >> 20) - e + 127;
@@ -380,7 +384,7 @@ __device__ __forceinline__ int species_vote_fp64(const double (&d)[4], double Wt
         for (int i = 0; i < wps; ++i) u += pf[(s * wps + i) * 4 + c];
         ok = u < l.lo;
         unsure = !ok && !(u > l.hi);
-            if (!__any_sync(kFull, unsure)) return ok;   // the same in every warp of the species
+        if (!__any_sync(kFull, unsure)) return ok;   // the same in every warp of the species
     }
     double v[4];
 #pragma unroll

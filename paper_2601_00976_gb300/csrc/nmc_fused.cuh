@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
     const double W2q = act ? g.w2[q] : 0.0;
     const double W3q = act ? g.w3[q] : 0.0;
     const R Wt = act ? (kMixed ? (R)g.wt_f[q] : (R)g.wt[q]) : (R)0;
-    const float Wt_f = act ? g.wt_f[q] : 0.0f;
+    const float Wt_f = act ? vote_weight(g.wt_f[q]) : 0.0f;
 
     // Mixed precision keeps the number moment D as a double-float (near a fixed
     // point where 1 + dtau chi ~ 1e4, FP32 increments of D fall below one ulp long

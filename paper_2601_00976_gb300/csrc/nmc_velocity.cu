@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(MAXT, MINB) velocity_kernel(const VelArgs va) 
     const double W2q = act ? g.w2[q] : 0.0;
     const double W3q = act ? g.w3[q] : 0.0;
     const double Wt = act ? g.wt[q] : 0.0;
-    const float Wt_f = act ? g.wt_f[q] : 0.0f;
+    const float Wt_f = act ? vote_weight(g.wt_f[q]) : 0.0f;
     double Fh[3][4], Qh[3][4];
     for (int j = 0; j < 3; ++j)
         for (int c = 0; c < 4; ++c) { Fh[j][c] = 0.0; Qh[j][c] = 0.0; }
