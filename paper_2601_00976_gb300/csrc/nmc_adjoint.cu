@@ -65,7 +65,7 @@ struct AdjNode {
     double ystar[2], y[2], yp[2], h[2];
     double deps_dT_star, deps_dYe_star;
     double g_y[2];           // cotangent of y = (eps, Ye): direct, through T_out and through kappa
-    double blk_out[8];
+    double blk_out[6];
     double dinv[128];        // reciprocals of the eliminated diagonal (2 ne <= 128)
     long long cv[2][8];      // per warp: bits of the largest |entry| of the next column among its active rows
     double cip[2][8];        //   (-1: none), its reciprocal,

@@ -687,12 +687,17 @@ struct OpacState {
     double eta_e;              // mu_e / T
     double mu[kMaxSpecies];    // neutrino chemical potentials per species
     double tinv;               // 1 / T
-    double w8[8], w4[4];       // corner weights of the EmAb/Iso cell (bits: rho, T, Ye) and the kernel cell (T, eta)
-    double pre[4];             // dtau sc_EmAb, dtau sc_Iso, and the NES and pair prefactors
-    // FP32 copies for the mixed-precision path: mu and 1 / T as double-floats
-    float mu_h[kMaxSpecies], mu_l[kMaxSpecies], tinv_h, tinv_l;
-    float w8_f[8], w4_f[4];
-    float pre_f[4];
+    union {                    // each precision's own
+        struct {
+            double w8[8], w4[4];   // corner weights of the EmAb/Iso cell (bits: rho, T, Ye) and the kernel cell (T, eta)
+            double pre[4];         // dtau sc_EmAb, dtau sc_Iso, and the NES and pair prefactors
+        };
+        struct {                   // mixed: mu and 1 / T as double-floats, the rest in FP32
+            float mu_h[kMaxSpecies], mu_l[kMaxSpecies], tinv_h, tinv_l;
+            float w8_f[8], w4_f[4];
+            float pre_f[4];
+        };
+    };
     int ir, it, iy, ikt, ike;  // table cells
 };
 

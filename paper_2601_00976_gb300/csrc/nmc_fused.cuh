@@ -78,8 +78,8 @@ struct NodeShared {
     float alpha_f[MAXM];
     VoteLimit lim[kMaxSpecies];   // Algorithm 2's thresholds (FP64 path)
     float t2_f[2][kMaxSpecies];   // square_thresholds for the D and I changes of the mixed path, from FP32 thresholds
-    double sp_out[kMaxSpecies * 4];
-    double blk_out[8];
+    double sp_out[kMaxSpecies];
+    double blk_out[2];
     OpacState op;
     long long node;
     int status, n_inner, n_outer;

@@ -57,8 +57,8 @@ struct VelNode {
     double G[3][3];
     double alpha[3];
     VoteLimit lim[kMaxSpecies];           // Algorithm 2's thresholds
-    double sp_out[kMaxSpecies * 4];
-    double blk_out[16];
+    double sp_out[kMaxSpecies];
+    double blk_out[kNsum];
     OpacState op;
     long long node;
     int status, n_inner, n_outer, conv_out, bad, done;
