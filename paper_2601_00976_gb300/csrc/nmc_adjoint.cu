@@ -67,9 +67,6 @@ struct AdjNode {
     double g_y[2];           // cotangent of y = (eps, Ye): direct, through T_out and through kappa
     double blk_out[6];
     double dinv[128];        // reciprocals of the eliminated diagonal (2 ne <= 128)
-    long long cv[2][8];      // per warp: bits of the largest |entry| of the next column among its active rows
-    double cip[2][8];        //   (-1: none), its reciprocal,
-    int ci[2][8];            //   and its row (double-buffered by column parity)
     int prow[128];           // pivot row of each eliminated column
     OpacState op;
 
@@ -367,6 +364,11 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                     // tracks, among the rows it has just updated, the largest |entry| of the next column
                     // (lane 0 updates that column), so one barrier per column publishes both the updated
                     // rows and the next pivot's candidates.  Every thread then picks the same pivot.
+                    // The candidates lie in the reduction scratch (64 bytes a warp, free here), one per warp and column
+                    // parity: the largest |entry|'s bits (-1: none), its reciprocal and its row.
+                    long long* cv = static_cast<long long*>(red);
+                    double* cip = reinterpret_cast<double*>(cv + 2 * nwarps);
+                    int* ci = reinterpret_cast<int*>(cip + 2 * nwarps);
                     // This warp's rows warp + nwarps i (at most 32 of them: 2 ne rows, ns nep >= 2 ne threads), those
                     // not yet a pivot row as a bit mask over i.
                     const int rows_w = (N2 - warp + nwarps - 1) / nwarps;
@@ -380,20 +382,20 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                             if (v > nb && v <= (long long)kInfBits) { nb = v; ni = r; }
                         }
                         if (nb > 0) nip = 1.0 / Mt[ni * LDM];
-                        nd->cv[0][warp] = nb;
-                        nd->ci[0][warp] = ni;
-                        nd->cip[0][warp] = nip;
+                        cv[warp] = nb;
+                        ci[warp] = ni;
+                        cip[warp] = nip;
                     }
                     __syncthreads();
                     for (int c = 0; c < N2; ++c) {
-                        const int bsel = c & 1;
+                        const int now = (c & 1) * nwarps, next = nwarps - now;
                         double ip = 0.0;
                         long long best = -1;
                         int P = 0;
                         for (int w = 0; w < nwarps; ++w) {
-                            const long long v = nd->cv[bsel][w];
-                            const int i = nd->ci[bsel][w];
-                            if (v > best || (v == best && i < P)) { best = v; P = i; ip = nd->cip[bsel][w]; }
+                            const long long v = cv[now + w];
+                            const int i = ci[now + w];
+                            if (v > best || (v == best && i < P)) { best = v; P = i; ip = cip[now + w]; }
                         }
                         if (best <= (long long)bits_of(1e-300) || best >= (long long)kInfBits) {   // singular: same decision in every thread
                             if (tid == lead) { nd->status |= NMC_NONFINITE; nd->bad = 1; }
@@ -446,9 +448,9 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
                         const int wrow = (int)__reduce_min_sync(kFull, (unsigned)(bkey == wkey && wkey >= 0 ? brow : 0x7fffffff));
                         if (lane == 0) {
                             const int ni = wkey >= 0 ? wrow : 0;
-                            nd->cv[bsel ^ 1][warp] = wkey;
-                            nd->ci[bsel ^ 1][warp] = ni;
-                            nd->cip[bsel ^ 1][warp] = wkey > 0 ? 1.0 / Mt[ni * LDM + c + 1] : 0.0;
+                            cv[next + warp] = wkey;
+                            ci[next + warp] = ni;
+                            cip[next + warp] = wkey > 0 ? 1.0 / Mt[ni * LDM + c + 1] : 0.0;
                         }
                         __syncthreads();
                     }
