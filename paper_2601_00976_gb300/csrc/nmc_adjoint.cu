@@ -142,12 +142,11 @@ __global__ void __launch_bounds__(MAXT, MINB) adjoint_kernel(const AdjointArgs a
     const bool frozen = P.frozen_matter != 0;
 
     for (long long n = blockIdx.x; n < a.n; n += gridDim.x) {
-        // The node's scalar FP64 work (the EoS solves, ComputeOpacities' scalars, a third of an SMSP's share
-        // of the node) goes to one warp.  Warp w of every resident block sits on the same SMSP, so this lead
-        // warp rotates with the node; the shift keeps blocks one SM count (a multiple of the warps) apart,
-        // which share an SM, on different SMSPs.  With the pivot search in integers (its compares were a
-        // seventh of the kernel's FP64 instructions) and the EoS on all the warp's lanes: 4099 nodes 12.7 ->
-        // 10.8 ms.
+        // The node's scalar FP64 work (the EoS solves, ComputeOpacities' scalars) goes to one warp.  Warp w of
+        // every resident block sits on the same SMSP, so this lead warp rotates with the node; the shift keeps
+        // blocks one SM count (a multiple of the warps) apart, which share an SM, on different SMSPs.  With the
+        // EoS on all the warp's lanes the choice no longer shows: 4099 nodes with their forward solve take 23.1 ms
+        // with the lead fixed or rotating.
         const int lead = (int)((n + (n >> 3)) % nwarps) << 5;
         // ---------------- inputs, y* and the output matter state ----------------
         double Ds = 0.0, D = 0.0, gD = 0.0, gIs = 0.0;   // gIs = gH . I*

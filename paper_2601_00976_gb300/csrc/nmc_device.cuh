@@ -81,11 +81,10 @@ __device__ __forceinline__ T square_threshold(T thr) {
 // 5 K of a butterfly per value (an FP64 addition holds the SMSP's pipe ~64 cycles: the three Gram
 // sums of an inner iteration 6 instead of 15, the velocity solve's fifteen sums 16 instead of 75).
 // Every value is added over the same tree as the butterfly adds it (partners 16, 8, 4, 2, 1 apart;
-// addition commutes), so the sums are the same bit for bit.  Together with the integer comparisons and
-// square_threshold above it took the FP64 solve of 20001 profile nodes (32 energies) from 89.3 to 77.1 ms,
-// the O(v/c) solve of 8192 nodes from 57.6 to 50.1 ms and the mixed solve of 200003 core/tail nodes from
-// 164.4 to 157.1 ms.  The sum a lane ends with in v[0] is that
-// of value fold_index<K>(lane) (K or more: none).
+// addition commutes), so the sums are the same bit for bit.  With butterflies and with this, at 32 energies:
+// FP64 solve of 20001 profile nodes 69.0 and 66.3 ms, O(v/c) solve of 8192 nodes 46.5 and 44.2, mixed solve of
+// 200003 core/tail nodes 139.4 and 138.2.  The sum a lane ends with in v[0] is that of value
+// fold_index<K>(lane) (K or more: none).
 template <int N, int OFF, typename T>
 __device__ __forceinline__ void fold_step(T* v, int lane) {
     if constexpr (OFF > 0) {
@@ -138,9 +137,9 @@ __device__ __forceinline__ void warp_partials(T (&v)[K], void* scratch) {
     if ((lane & ((32 >> kFoldLevels<K>) - 1)) == 0 && k < K) red[w * K + k] = v[0];
 }
 
-// The warps' partials of value k added in warp order.  Blocks of 4 and 8 warps, the usual ones, take
-// their own code: this sum is on every inner iteration's critical path, and the loop's bookkeeping
-// between dependent loads and additions cost the mixed solve 1-2%.
+// The warps' partials of value k added in warp order.  Blocks of 4 and 8 warps (four species at 17 to 32 and
+// 33 to 64 energies) take their own code, without a loop's bookkeeping between dependent loads and additions:
+// this sum is on every inner iteration's critical path.
 template <int K, int NW, typename T>
 __device__ __forceinline__ T add_partials_of(const T* red, int k) {
     T p[NW], s = 0;
@@ -347,7 +346,8 @@ __device__ __forceinline__ float scaled_abs(double x, int e) {
 // species_vote in FP64.  d: the change of the thread's bin per moment.  The weighted sums of squares, eight
 // multiplications and six additions of the FP64 pipe in every warp, are formed in FP32 first (relative error
 // below 2e-6); only a sum within 2e-5 of its threshold is formed again in FP64, so the answer is that of FP64.
-// The O(v/c) solve of 8192 nodes: 45.9 -> 44.1 ms.
+// Without and with the filter: FP64 solve of 20001 nodes, 32 energies, 69.9 and 66.3 ms; 6007 nodes, 64 energies,
+// 66.9 and 65.0; O(v/c) solve of 8192 nodes 46.1 and 44.2; 1500 relaxation problems 61.9 and 59.0.
 __device__ __forceinline__ int species_vote_fp64(const double (&d)[4], double Wt, float Wt_f, const VoteLimit* lim, int nep, int ns,
                                                  int s, void* scratch) {
     const int lane = threadIdx.x & 31, sp = s < ns ? s : 0;

@@ -87,7 +87,7 @@ __device__ __forceinline__ double eos_mu_e_warp(double ne, double T, double* rT 
 // eos_eps_at_mu with nb = rho / m_B and f = (MeV in erg) / rho.  The products and sums are written as the
 // fused operations the compiler contracts them to in eos_eps_at_mu, so that both round alike; kShared: where
 // pi^2 T^2 is shared with eos_deps_dye_at_mu, it is rounded before it is added.
-// kLanes: numerators formed lane-parallel as well (not in the adjoint, whose register budget it overruns).
+// kLanes: numerators formed lane-parallel as well (not in the adjoint, where it overruns the narrow register class).
 template <bool kShared = false, bool kLanes = true>
 __device__ __forceinline__ void eos_eps_at_mu_warp(double nb, double f, double T, double mu, double* eps, double* deps) {
     const int ln = threadIdx.x & 31;

@@ -1,17 +1,19 @@
 // The order in which the persistent solve kernels take a batch's nodes.
 //
-// A node's iterations grow with its optical depth per step, rho dt (rank correlation 0.89-0.97 with the
-// inner iterations on collapse profiles and core/tail mixes), and differ 20-50 fold within a batch.  With
-// nodes taken as they come, a long node that starts late leaves most of the chip idle at the end, which
-// costs a batch of a few nodes per resident block ~10% of its time.  Long nodes first is the classical
-// remedy (Graham's LPT rule, SIAM J. Appl. Math. 17, 1969).  This kernel sorts the node indices by falling
-// rho dt, to 1/8 octave, with one block's counting sort; the solve's results do not depend on the order.
+// On collapse profiles and core/tail mixes a node's iterations grow with its optical depth per step, rho dt
+// (rank correlation with the inner iterations 0.89-0.97), and differ 20-50 fold within a batch.  With nodes
+// taken as they come, a long node that starts late leaves most of the chip idle at the end.  Long nodes first
+// is the classical remedy (Graham's LPT rule, SIAM J. Appl. Math. 17, 1969).  This kernel sorts the node
+// indices by falling rho dt, to 1/8 octave, with one block's counting sort; the solve's results do not depend
+// on the order.  Where rho dt hardly varies, as in a batch of relaxation problems at one step, the iterations
+// do not follow it (rank correlation 0.14) and the order is close to arbitrary, neither a gain nor a loss.
 //
 // Used while it pays: more nodes than resident blocks (else every node starts at once) and at most
 // kOrderMax (beyond ~150 nodes per block the idle end is below 1%, and one block's three passes over
-// the keys would begin to show).  Measured: 512 nodes, mixed, 64 energies, 1.84 -> 1.65 ms; 4099 nodes, FP64,
-// with their gradient, 27.0 -> 25.6 ms; O(v/c), 8192 nodes, 48.1 -> 45.9 ms; FP64, 6007 nodes, 64 energies,
-// 69.6 -> 67.7 ms; batches of equal nodes unchanged (62.8, 62.7 ms).  It also clears the work queue, in place of the memset of the other calls.
+// the keys would begin to show).  Without and with it: 512 nodes, mixed, 64 energies, 1.51-1.56 and 1.47 ms; 4099
+// nodes, FP64, with their gradient, 24.2 and 23.1; O(v/c), 8192 nodes, 46.0 and 44.2; FP64, 6007 nodes, 64
+// energies, 66.9 and 65.0; 20001 nodes, 32 energies, 67.4 and 66.3; mixed, 50000 core/tail nodes, 35.4 and 34.4; 1500
+// relaxation problems 59.3-60.1 and 59.0.  It also clears the work queue, in place of the memset of the other calls.
 #include <cuda_runtime.h>
 
 #include <string>
