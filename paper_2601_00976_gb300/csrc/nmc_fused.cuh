@@ -226,8 +226,9 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
         // components then stay zero through the whole solve: their 22 FP64 instructions of an inner iteration
         // are left out.  The same nodes with and without the branch: 20001 nodes, 32 energies, 67.7 -> 66.2 ms; 6007
         // nodes, 64 energies, 66.1 -> 65.2 ms (with flux in all directions 67.6 and 66.1 ms).  A first component that
-        // is not finite, or so large that its product with 1 / (1 + dtau kappa) could overflow, takes the general
-        // form, so that a non-finite product can only come from that factor (below).
+        // is not finite, or so large that a product with 1 / (1 + dtau kappa) or a coefficient could overflow, takes
+        // the general form, so that a non-finite result can only come from that factor (at the node's end: inside
+        // the iteration the test cost 0.5% of one node's latency).
         const bool flux3 = __syncthreads_or(kMixed || MAXM != 3 || (bits_of(Isd[1]) << 1) != 0 || (bits_of(Isd[2]) << 1) != 0 ||
                                             exponent_of(Isd[0]) > 1023 + 500) != 0;
         if (nd->done) {   // invalid input: outputs = inputs
@@ -610,11 +611,8 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                     }
                     if constexpr (kMixed) v[0] = Wt * sD * sD;
                     if (act && !(is_finite(Mn[0]) && is_finite(Mn[1]) && is_finite(Mn[2]) && is_finite(Mn[3]) &&
-                                 is_finite(sD))) {
+                                 is_finite(sD)))
                         nd->bad = 1;
-                        // a factor 1 / (1 + dtau kappa) that is not finite makes NaN of the zero components as well
-                        if (!kMixed && !flux3 && !is_finite(Qv[1])) Mn[2] = Mn[3] = (R)__longlong_as_double(0x7ff8000000000000ll);
-                    }
                     // the scratch is free here: the lead warp read the Gram partials before the previous
                     // barrier, and the next ones are written after the vote's
                     if constexpr (kMixed) vote = species_vote(v, nd->t2_f[0], nd->t2_f[1], NEP, NS, s, red);
@@ -725,6 +723,8 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
                 a.status[n] = (uint32_t)st;
             }
         }
+        // a factor 1 / (1 + dtau kappa) that is not finite makes NaN of the zero components as well
+        if (!flux3 && !is_finite(M[1])) M[2] = M[3] = (R)__longlong_as_double(0x7ff8000000000000ll);
         if (act && NMC_IN_BOUNDS(g.dbg, (n * NS + s) * NE + q, a.n * NS * NE, kDbgOutput)) {
             const long long o = (n * NS + s) * NE + q;
             a.J_out[o] = kMixed ? f2_to(Dx) : (double)M[0];
