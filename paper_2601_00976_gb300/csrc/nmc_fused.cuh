@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(MAXT, MINB) fused_kernel(const SolveArgs a) {
             }
         }
         // a factor 1 / (1 + dtau kappa) that is not finite makes NaN of the zero components as well
-        if (!flux3 && !is_finite(M[1])) M[2] = M[3] = (R)__longlong_as_double(0x7ff8000000000000ll);
+        if (!kMixed && !flux3 && !is_finite(M[1])) M[2] = M[3] = (R)__longlong_as_double(0x7ff8000000000000ll);
         if (act && NMC_IN_BOUNDS(g.dbg, (n * NS + s) * NE + q, a.n * NS * NE, kDbgOutput)) {
             const long long o = (n * NS + s) * NE + q;
             a.J_out[o] = kMixed ? f2_to(Dx) : (double)M[0];
